@@ -29,16 +29,16 @@ static cudaError_t launch_conv_full_blk(const RowArgs<W> &a, int grid, cudaStrea
 {
     constexpr int RW = Arith<W>::RB + 5;
     if constexpr (L <= RW) {
-        constexpr size_t smem = TwBytes<W, L>::v + RowShape<W, L, L, BLK>::smem(2);
+        constexpr size_t smem = FusedShape<W, L, BLK>::smem;
         static const cudaError_t init = ensure_smem(k_conv_fused<W, L, SRC, BLK>, smem);
         if (init != cudaSuccess) return init;
         k_conv_fused<W, L, SRC, BLK><<<grid, BLK, smem, st>>>(a);
         return launched();
     } else if constexpr (L <= LRMax<W>::v && (BLK == BLOCK || L < LRMax<W>::v)) {
-        constexpr size_t smem = CRShape<W, L, L, BLK>::smem;
-        static const cudaError_t init = ensure_smem(k_conv_cr<W, L, L, SRC, 0, BLK>, smem);
+        constexpr size_t smem = CRShape<W, L, true, BLK>::smem;
+        static const cudaError_t init = ensure_smem(k_conv_cr<W, L, SRC, 0, BLK>, smem);
         if (init != cudaSuccess) return init;
-        k_conv_cr<W, L, L, SRC, 0, BLK><<<grid, BLK, smem, st>>>(a);
+        k_conv_cr<W, L, SRC, 0, BLK><<<grid, BLK, smem, st>>>(a);
         return launched();
     } else {
         return cudaErrorInvalidValue;
@@ -63,8 +63,8 @@ template <typename W, int L>
 static size_t full_smem_of()
 {
     constexpr int RW = Arith<W>::RB + 5;
-    if constexpr (L <= RW) return TwBytes<W, L>::v + RowShape<W, L, L>::smem(2);
-    else if constexpr (L <= LRMax<W>::v) return CRShape<W, L>::smem;
+    if constexpr (L <= RW) return FusedShape<W, L>::smem;
+    else if constexpr (L <= LRMax<W>::v) return CRShape<W, L, true>::smem;
     else return 0;
 }
 
@@ -133,15 +133,15 @@ static cudaError_t launch_conv_rows(bool twisted, const RowArgs<W> &a, int grid,
     constexpr int LR = LRMax<W>::v;
     if constexpr (L > LR && L <= Launch<W>::LMAX) {
         if (twisted) {
-            constexpr size_t smem = CRShape<W, LR, LR>::smem;
-            static const cudaError_t init = ensure_smem(k_conv_cr<W, LR, LR, 0, 1>, smem);
+            constexpr size_t smem = CRShape<W, LR, true>::smem;
+            static const cudaError_t init = ensure_smem(k_conv_cr<W, LR, 0, 1>, smem);
             if (init != cudaSuccess) return init;
-            k_conv_cr<W, LR, LR, 0, 1><<<grid, BLOCK, smem, st>>>(a);
+            k_conv_cr<W, LR, 0, 1><<<grid, BLOCK, smem, st>>>(a);
         } else {
-            constexpr size_t smem = CRShape<W, L, LR>::smem;
-            static const cudaError_t init = ensure_smem(k_conv_cr<W, L, LR, 0>, smem);
+            constexpr size_t smem = CRShape<W, LR, false>::smem;
+            static const cudaError_t init = ensure_smem(k_conv_rows<W, L, LR>, smem);
             if (init != cudaSuccess) return init;
-            k_conv_cr<W, L, LR, 0><<<grid, BLOCK, smem, st>>>(a);
+            k_conv_rows<W, L, LR><<<grid, BLOCK, smem, st>>>(a);
         }
         return launched();
     } else {

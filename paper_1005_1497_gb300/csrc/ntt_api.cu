@@ -94,9 +94,10 @@ struct ntt_plan_s {
     int block = ntt::BLOCK;            // whole sequences: threads per block of the fused kernel
     long long small_max = 0;           // whole one-warp lengths: batches up to this run one block per pair
     void *scratch = nullptr;           // 2 * wave * N words
-    void *pw = nullptr;                // split path: (w^e, Shoup quotient), e < N (the twist)
-    void *pd = nullptr;                // one column pass: the twist factor of element x, at x (the diagonal)
-    void *pwl = nullptr;               // split path: (w^(s l), quotient) at s 32 + l, s < 2^(L - LR), l < 32
+    void *pd = nullptr;                // split path, one column pass: the scaled twist factor of element x, at x
+    void *pw = nullptr;                // split path, two column passes: (w^e, Shoup quotient), e < N
+    void *pwl = nullptr;               // and (scaled w^(s l), quotient) at s 32 + l, s < 2^(L - LR), l < 32
+    uint64_t twist_unscale = 1;        // inverse of the scale that the twist's factors carry
     int nsm = 1;
     int device = 0;
     unsigned long long *counter = nullptr;
@@ -120,6 +121,9 @@ static void fill_modc(ModC<W> &c, uint64_t m, uint64_t ninv)
     c.onep = (W)nt::shoup_quot(1, m, B);
     c.ninv = (W)ninv;
     c.ninvp = (W)nt::shoup_quot(ninv, m, B);
+    const uint64_t cB = nt::shl_mod(cN, ntt::BB, m);
+    c.cB = (W)cB;
+    c.cBp = (W)nt::shoup_quot(cB, m, B);
 }
 
 static int num_sms()
@@ -231,55 +235,51 @@ extern "C" ntt_status ntt_plan(uint64_t m, uint32_t N, ntt_plan_t *out)
         if (wave < 1) wave = 1;
         p->wave = (uint32_t)wave;
         if (!ntt::dev_alloc(&p->scratch, 2 * wave * N * elt)) return ntt_fail(NTT_ERR_OOM, "ntt_plan: scratch");
-        // powers w^e, e < N, for the twist between the column and row passes
-        // (w^e = 2^{e N_Max / N}, again from the doubling sequence)
-        std::vector<uint64_t> all = nt::powers_of_two_by_doubling((nmax / N) * (uint64_t)N, m);
+        // Factors of the twist between the column and row passes: powers of w
+        // (again from the doubling sequence: w^e = 2^{e N_Max / N}) times a
+        // scale s.  The row kernel convolves by blocks and leaves out the
+        // factor 2^(B + BB) / N (ntt_block.cuh); an element's path to its
+        // output meets the twist three times (f's, g's and the inverse one),
+        // so every factor carries s = 2^((B + BB - L) / 3), the division
+        // modulo N_Max: a power of two has exactly one cube root among them.
+        // (The row-twiddle form does not use these tables.)
+        const std::vector<uint64_t> all = nt::powers_of_two_by_doubling(nmax, m);
+        const uint64_t third = nmax % 3 == 1 ? (2 * nmax + 1) / 3 : (nmax + 1) / 3;    // 3^-1 mod N_Max
+        const uint64_t se = (uint64_t)(B + ntt::BB - L) * third % nmax;
+        p->twist_unscale = all[(nmax - se) % nmax];
         std::vector<unsigned char> tab(2 * (size_t)N * elt);
-        for (size_t e = 0; e < N; ++e) {
-            const uint64_t z = all[e * (nmax / N)], zp = nt::shoup_quot(z, m, B);
+        auto put = [&](std::vector<unsigned char> &t, size_t i, uint64_t z) {
             if (word == 32) {
-                uint32_t a[2] = {(uint32_t)z, (uint32_t)zp};
-                memcpy(&tab[2 * e * elt], a, sizeof a);
+                const uint32_t a[2] = {(uint32_t)z, (uint32_t)((z << 32) / m)};
+                memcpy(&t[2 * i * elt], a, sizeof a);
             } else {
-                uint64_t a[2] = {z, zp};
-                memcpy(&tab[2 * e * elt], a, sizeof a);
+                const uint64_t a[2] = {z, nt::shoup_quot(z, m, B)};
+                memcpy(&t[2 * i * elt], a, sizeof a);
             }
-        }
-        if (!ntt::dev_alloc(&p->pw, tab.size())) return ntt_fail(NTT_ERR_OOM, "ntt_plan: power table");
-        CUDA_TRY(cudaMemcpy(p->pw, tab.data(), tab.size(), cudaMemcpyHostToDevice), "ntt_plan: upload powers");
+        };
         if (L - p->LR <= 5) {
             // one column pass: element x = t + k 2^LR (t < 2^LR, k < 2^(L-LR))
-            // takes w^(brv(k) t), the same for every pair, so the factor is
+            // takes s w^(brv(k) t), the same for every pair, so the factor is
             // stored at x and read in the data's own (coalesced) layout
             const int lc = L - p->LR;
-            std::vector<unsigned char> dg(tab.size());
             for (size_t x = 0; x < N; ++x) {
                 const size_t k = x >> p->LR, t = x & (((size_t)1 << p->LR) - 1);
-                size_t sk = 0;
-                for (int i = 0; i < lc; ++i) sk |= ((k >> i) & 1u) << (lc - 1 - i);
-                const size_t e = (sk * t) % N;
-                memcpy(&dg[2 * x * elt], &tab[2 * e * elt], 2 * elt);
+                put(tab, x, all[((nt::bit_reverse(k, lc) * t) % N * (nmax / N) + se) % nmax]);
             }
-            if (!ntt::dev_alloc(&p->pd, dg.size())) return ntt_fail(NTT_ERR_OOM, "ntt_plan: twist diagonal");
-            CUDA_TRY(cudaMemcpy(p->pd, dg.data(), dg.size(), cudaMemcpyHostToDevice), "ntt_plan: upload twist diagonal");
+            if (!ntt::dev_alloc(&p->pd, tab.size())) return ntt_fail(NTT_ERR_OOM, "ntt_plan: twist diagonal");
+            CUDA_TRY(cudaMemcpy(p->pd, tab.data(), tab.size(), cudaMemcpyHostToDevice), "ntt_plan: upload twist diagonal");
+        } else {
+            // two column passes: w^e for e < N, and s w^(s l) per lane
+            for (size_t e = 0; e < N; ++e) put(tab, e, all[e * (nmax / N)]);
+            if (!ntt::dev_alloc(&p->pw, tab.size())) return ntt_fail(NTT_ERR_OOM, "ntt_plan: power table");
+            CUDA_TRY(cudaMemcpy(p->pw, tab.data(), tab.size(), cudaMemcpyHostToDevice), "ntt_plan: upload powers");
+            const size_t ns = (size_t)1 << (L - p->LR);
+            std::vector<unsigned char> lt(2 * ns * 32 * elt);
+            for (size_t sidx = 0; sidx < ns; ++sidx)
+                for (size_t l = 0; l < 32; ++l) put(lt, sidx * 32 + l, all[((sidx * l) % N * (nmax / N) + se) % nmax]);
+            if (!ntt::dev_alloc(&p->pwl, lt.size())) return ntt_fail(NTT_ERR_OOM, "ntt_plan: lane power table");
+            CUDA_TRY(cudaMemcpy(p->pwl, lt.data(), lt.size(), cudaMemcpyHostToDevice), "ntt_plan: upload lane powers");
         }
-        const size_t ns = (size_t)1 << (L - p->LR);
-        std::vector<unsigned char> lt(2 * ns * 32 * elt);
-        for (size_t sidx = 0; sidx < ns; ++sidx)
-            for (size_t l = 0; l < 32; ++l) {
-                const uint64_t e = (sidx * l) % N;
-                const uint64_t z = all[e * (nmax / N)], zp = nt::shoup_quot(z, m, B);
-                const size_t i = sidx * 32 + l;
-                if (word == 32) {
-                    uint32_t a[2] = {(uint32_t)z, (uint32_t)zp};
-                    memcpy(&lt[2 * i * elt], a, sizeof a);
-                } else {
-                    uint64_t a[2] = {z, zp};
-                    memcpy(&lt[2 * i * elt], a, sizeof a);
-                }
-            }
-        if (!ntt::dev_alloc(&p->pwl, lt.size())) return ntt_fail(NTT_ERR_OOM, "ntt_plan: lane power table");
-        CUDA_TRY(cudaMemcpy(p->pwl, lt.data(), lt.size(), cudaMemcpyHostToDevice), "ntt_plan: upload lane powers");
     }
     *out = p.release();
     return NTT_OK;
@@ -376,7 +376,11 @@ static cudaError_t ntt_dispatch(ntt_plan_t p, const W *x, W *y, long long batch,
         const int grid = row_grid(p->nsm, rows, Launch<W>::rows_per_block(p->LR));
         e = twisted ? Launch<W>::rows_uni(ra, grid, st) : Launch<W>::rows_fwd(p->L, ra, grid, st);
         if (e != cudaSuccess) return e;
-        e = Launch<W>::bitrev_out(p->L, inv, scratch, y + (size_t)w0 * N, np, c, st);
+        ModC<W> cs = c;                                // the output factor: N^-1, and the twist's scale undone
+        const uint64_t sc = nt::mul_mod(inv ? p->n_inv : 1, twisted ? p->twist_unscale : 1, p->m);
+        cs.ninv = (W)sc;
+        cs.ninvp = (W)nt::shoup_quot(sc, p->m, (int)sizeof(W) * 8);
+        e = Launch<W>::bitrev_out(p->L, inv, scratch, y + (size_t)w0 * N, np, cs, st);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;

@@ -68,6 +68,8 @@ template <typename W> struct ModC {
     W onep;     // floor(2^B / m): Shoup quotient of the factor 1
     W ninv;     // N^{-1} mod m
     W ninvp;    // floor(ninv 2^B / m)
+    W cB;       // 2^BB N^{-1} 2^B mod m: the last factor of a convolution by blocks (ntt_block.cuh)
+    W cBp;      // floor(cB 2^B / m)
 };
 
 // Shoup product: b z mod m in [0, 2m) for any b < 2^B, given zp = floor(z 2^B / m).
@@ -76,6 +78,20 @@ __device__ __forceinline__ W shoup(W b, W z, W zp, W m)
 {
     W q = Arith<W>::mulhi(b, zp);
     return b * z - q * m;
+}
+
+// 32-bit words: the three products as written, the second accumulating onto
+// the first (nvcc otherwise reassociates them into the butterfly's sums).
+// Measured on GB300 in a loop of butterflies on registers: 8.8 -> 8.4 cycles
+// per butterfly and scheduler (8 is the multiply pipe's limit).
+template <>
+__device__ __forceinline__ uint32_t shoup<uint32_t>(uint32_t b, uint32_t z, uint32_t zp, uint32_t m)
+{
+    uint32_t q, t, r;
+    asm("mul.hi.u32 %0, %1, %2;" : "=r"(q) : "r"(b), "r"(zp));
+    asm("mul.lo.u32 %0, %1, %2;" : "=r"(t) : "r"(b), "r"(z));
+    asm("mad.lo.u32 %0, %1, %2, %3;" : "=r"(r) : "r"(q), "r"(0u - m), "r"(t));
+    return r;
 }
 
 // v in [0, 2m) -> [0, m)
@@ -275,7 +291,8 @@ __device__ __forceinline__ void stage_twiddles(const W *__restrict__ tw, W *stw,
 // leaves < 2m and every node-0 butterfly of levels 1..4 doubles the bound
 // (< 2^(d+1) m after level d), the others add 2m: at most 32m + 2m (L - 5)
 // after the forward, below 50m for L <= 14.
-template <typename W, int L, int LR, int P, int JJ, int NS, int TWS, bool Z0 = false>
+// UN: the last level whose node 0 skips the product.
+template <typename W, int L, int LR, int P, int JJ, int NS, int TWS, bool Z0 = false, int UN = 4>
 __device__ __forceinline__ void fwd_level(W (&v)[NS][Geo<W, LR>::R], uint32_t xbase,
                                           const W *__restrict__ tw, const ModC<W> &c)
 {
@@ -293,7 +310,7 @@ __device__ __forceinline__ void fwd_level(W (&v)[NS][Geo<W, LR>::R], uint32_t xb
     } else {
         constexpr int CNT = R >> (JJ + 1);      // distinct nodes touched by this thread
         constexpr int CH = (CNT >= 2 && tw_per_chunk<W>() == 2) ? 2 : 1;
-        constexpr bool UNIT0 = Z0 && P == 0 && dg <= 4;
+        constexpr bool UNIT0 = Z0 && P == 0 && dg <= UN;
         const uint32_t nb = xbase >> (b + 1);   // aligned to CNT
 #pragma unroll
         for (int t0 = 0; t0 < CNT; t0 += CH) {

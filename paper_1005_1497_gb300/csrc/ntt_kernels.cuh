@@ -2,7 +2,9 @@
 // the word type W (uint32_t / uint64_t) and on log2 N.
 #pragma once
 
-#include "ntt_core.cuh"
+#include <type_traits>
+
+#include "ntt_block.cuh"
 #include "ntt_exact.cuh"
 
 namespace ntt {
@@ -55,6 +57,19 @@ struct RowShape {
     static constexpr size_t smem(int ns) { return (size_t)GPC * ns * G::ROWP * sizeof(W); }
 };
 
+// Shared memory of the one-warp fused kernel: the twiddles (the first N / 8
+// pairs for lengths that convolve by blocks) and, for lengths of more than
+// one register pass, two rows per group.
+template <typename W, int L, int BLK = BLOCK>
+struct FusedShape {
+    static constexpr bool BLOCKS = L >= BLOCK_LMIN;
+    using G = BGeo<W, L>;
+    static constexpr int GPC = BLK / G::T;
+    static constexpr int TWL = BLOCKS ? L - BB : L;     // TwBytes: 2^(TWL - 1) pairs
+    static constexpr int GS = G::NPASS > 1 ? G::GS : 0;
+    static constexpr size_t smem = TwBytes<W, TWL>::v + (size_t)GPC * GS * sizeof(W);
+};
+
 // Hint: fetch `bytes` bytes at p into L2 with one bulk copy-engine
 // request (no registers, no shared memory).  Skipped unless 16-byte aligned.
 __device__ __forceinline__ void prefetch_l2(const void *p, uint32_t bytes)
@@ -62,6 +77,17 @@ __device__ __forceinline__ void prefetch_l2(const void *p, uint32_t bytes)
     if (((uintptr_t)p & 15u) == 0 && bytes >= 16)
         asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes & ~15u) : "memory");
 }
+
+// Asynchronous copies into shared memory, and the wait for all of this
+// thread's (visible to others after the next barrier).
+template <int BYTES>
+__device__ __forceinline__ void cp_async(void *dst, const void *src)
+{
+    const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
+    if constexpr (BYTES == 16) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
+    else asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(d), "l"(src), "n"(BYTES) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 // Input and output of the fused bodies: plain words (the default), or the
 // ends of the exact convolution fused in -- signed 64-bit inputs reduced
@@ -109,27 +135,29 @@ __device__ __forceinline__ void st_out(W *hp, long long pair, uint32_t N, uint32
 // Fused convolution of whole sequences (L <= LR_max), persistent.  The block
 // stages the twiddle table in shared memory once.  Per pair, f and g are
 // transformed together (one set of twiddle reads serves both) through shared
-// regions 0 and 1, multiplied pointwise, and sent back through region 0 by
-// the decimation-in-time inverse; results are stored canonical at <-x>_N.
+// regions 0 and 1, multiplied block by block (ntt_block.cuh; lengths below 8
+// pointwise), and sent back through region 0 by the decimation-in-time
+// inverse; results are stored canonical.
 // At the start of each pair one thread asks the copy engine to bring the
 // next pair's f and g into L2, so their loads do not wait on HBM.
 // Rows [base + group, a.nrows) by steps of stride.
-template <typename W, int L, int SRC, class X = NoExact>
+template <typename W, int L, int SRC, class X = NoExact, int BLK = BLOCK>
 __device__ __forceinline__ void conv_fused_body(const RowArgs<W> &a, long long base, long long stride,
                                                 const ExactArgs *xa = nullptr)
 {
     using G = Geo<W, L>;
-    constexpr int T = G::T, R = G::R, GPC = RowShape<W, L, L>::GPC;
+    using SH = FusedShape<W, L, BLK>;
+    constexpr int T = G::T, R = G::R;
     constexpr uint32_t N = 1u << L;
     constexpr int last = G::NPASS - 1;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int gid = threadIdx.x / T;
     const uint32_t tau = threadIdx.x % T;
     W *stw = reinterpret_cast<W *>(smem_raw);
-    W *S = reinterpret_cast<W *>(smem_raw + TwBytes<W, L>::v) + (size_t)gid * 2 * G::ROWP;
+    W *S = reinterpret_cast<W *>(smem_raw + TwBytes<W, SH::TWL>::v) + (size_t)gid * SH::GS;
     const uint32_t b0 = G::base(0, tau);
     constexpr int lo0 = G::lo(0);
-    stage_twiddles<W>(a.tw, stw, TwBytes<W, L>::pairs);
+    stage_twiddles<W>(a.tw, stw, TwBytes<W, SH::TWL>::pairs);
     __syncthreads();
 
     auto ptrs = [&](long long rho, const W *&fp, const W *&gp, W *&hp) {
@@ -160,14 +188,23 @@ __device__ __forceinline__ void conv_fused_body(const RowArgs<W> &a, long long b
             v[0][k] = ld_elem<X>(fp, b0 + ((uint32_t)k << lo0), xa);
             v[1][k] = ld_elem<X>(gp, b0 + ((uint32_t)k << lo0), xa);
         }
-        fwd_all<W, L, L, 0, 2, TW_SMEM, true>(v, 0u, tau, S, gid, stw, a.c);
+        if constexpr (SH::BLOCKS) {
+            bfwd_all<W, L, L, 0, true>(v, 0u, tau, S, gid, stw, a.c);
+            block_products<W, R>(v, G::base(last, tau), stw, a.c);
+            bdit_all<W, L, last>(v[0], tau, S, gid, stw, a.c);
 #pragma unroll
-        for (int k = 0; k < R; ++k) v[0][k] = pointwise(v[0][k], v[1][k], a.c);
-        dit_all<W, L, last, TW_SMEM>(v[0], 0u, tau, S, gid, stw, a.c);
+            for (int k = 0; k < R; ++k) {
+                const uint32_t x = b0 + ((uint32_t)k << lo0);
+                st_out<X>(hp, a.pair0 + rho, N, block_out<L>(x), canon<W>(v[0][k], a.c.cB, a.c.cBp, a.c.m), xa);
+            }
+        } else {                                            // one thread per pair, no exchange
+            fwd_all<W, L, L, 0, 2, TW_SMEM, true>(v, 0u, tau, S, gid, stw, a.c);
 #pragma unroll
-        for (int k = 0; k < R; ++k) {
-            const uint32_t x = b0 + ((uint32_t)k << lo0);
-            st_out<X>(hp, a.pair0 + rho, N, (N - x) & (N - 1u), canon<W>(v[0][k], (W)1, a.c.onep, a.c.m), xa);
+            for (int k = 0; k < R; ++k) v[0][k] = pointwise(v[0][k], v[1][k], a.c);
+            dit_all<W, L, last, TW_SMEM>(v[0], 0u, tau, S, gid, stw, a.c);
+#pragma unroll
+            for (int k = 0; k < R; ++k)
+                st_out<X>(hp, a.pair0 + rho, N, (N - (uint32_t)k) & (N - 1u), canon<W>(v[0][k], (W)1, a.c.onep, a.c.m), xa);
         }
     }
 }
@@ -175,8 +212,8 @@ __device__ __forceinline__ void conv_fused_body(const RowArgs<W> &a, long long b
 template <typename W, int L, int SRC, int BLK = BLOCK>
 __global__ void __launch_bounds__(BLK, BLOCK / BLK) k_conv_fused(const __grid_constant__ RowArgs<W> a)
 {
-    constexpr int GPC = RowShape<W, L, L, BLK>::GPC;
-    conv_fused_body<W, L, SRC>(a, (long long)blockIdx.x * GPC, (long long)gridDim.x * GPC);
+    constexpr int GPC = FusedShape<W, L, BLK>::GPC;
+    conv_fused_body<W, L, SRC, NoExact, BLK>(a, (long long)blockIdx.x * GPC, (long long)gridDim.x * GPC);
 }
 
 // ---- column/row fused kernel ---------------------------------------------
@@ -225,8 +262,8 @@ __device__ __forceinline__ void colf_levels(W (&v)[RR], uint32_t rowbase, const 
 #pragma unroll
                     for (int j = 0; j < (1 << J); ++j) {
                         const int k = ((t0 + tt) << (J + 1)) | j;
-                        // whole sequence: node 0 has the twiddle 1 (bound note at fwd_level)
-                        if (DG0 == 0 && dg <= 4 && t0 + tt == 0) ct_bfly_unit<W>(v[OFF + k], v[OFF + (k | (1 << J))], c.m << dg);
+                        // whole sequence: node 0 has the twiddle 1 (bounds: ntt_block.cuh)
+                        if (DG0 == 0 && dg <= 2 && t0 + tt == 0) ct_bfly_unit<W>(v[OFF + k], v[OFF + (k | (1 << J))], c.m << dg);
                         else ct_bfly<W>(v[OFF + k], v[OFF + (k | (1 << J))], z[tt], zp[tt], c);
                     }
             }
@@ -280,33 +317,6 @@ __device__ __forceinline__ void colg_all(W (&v)[RR], uint32_t rowbase, const W *
     }
 }
 
-// Inverse (decimation-in-time) levels l = RW + J of one column c, tlo = brv_RW(c).
-template <typename W, int LC, int OFF, int J, int TWS, int RR>
-__device__ __forceinline__ void cold_levels(W (&v)[RR], uint32_t tlo, const W *__restrict__ tw, const ModC<W> &c)
-{
-    if constexpr (J < LC) {
-        constexpr int RC = 1 << LC;
-        constexpr int CNT = 1 << J;
-        constexpr int CH = (CNT >= 2 && tw_per_chunk<W>() == 2) ? 2 : 1;
-        const uint32_t run = tlo << J;
-#pragma unroll
-        for (int t0 = 0; t0 < CNT; t0 += CH) {
-            W z[CH], zp[CH];
-            load_tw<W, CH, TWS>(tw, run, (uint32_t)t0, z, zp);
-#pragma unroll
-            for (int tt = 0; tt < CH; ++tt) {
-                const int j = brv_c<J>(t0 + tt);
-#pragma unroll
-                for (int hi = 0; hi < (RC >> (J + 1)); ++hi) {
-                    const int k = (hi << (J + 1)) | j;
-                    ct_bfly<W>(v[OFF + k], v[OFF + (k | (1 << J))], z[tt], zp[tt], c);
-                }
-            }
-        }
-        cold_levels<W, LC, OFF, J + 1, TWS, RR>(v, tlo, tw, c);
-    }
-}
-
 // All columns JC .. CPT-1 held by a thread (column j at v[j * 2^LC ..]).
 template <typename W, int LC, int JC, int CPT, int DG0, int TWS, int RR>
 __device__ __forceinline__ void colf_all(W (&v)[RR], uint32_t rowbase, const W *__restrict__ tw, const ModC<W> &c)
@@ -317,69 +327,111 @@ __device__ __forceinline__ void colf_all(W (&v)[RR], uint32_t rowbase, const W *
     }
 }
 
-template <typename W, int LC, int RW, int JC, int CPT, int TPP, int TWS, int RR>
-__device__ __forceinline__ void cold_all(W (&v)[RR], uint32_t ptau, const W *__restrict__ tw, const ModC<W> &c)
+template <typename W, int LC, int RW, int VEC, int TPP, int JC, int NV, int RR>
+__device__ __forceinline__ void bcold_all(W (&v)[RR], uint32_t ptau, const W *__restrict__ tw, const ModC<W> &c)
 {
-    if constexpr (JC < CPT) {
-        const uint32_t col = ptau + (uint32_t)JC * TPP;
-        cold_levels<W, LC, JC * (1 << LC), 0, TWS, RR>(v, __brev(col) >> (32 - RW), tw, c);
-        cold_all<W, LC, RW, JC + 1, CPT, TPP, TWS, RR>(v, ptau, tw, c);
+    if constexpr (JC < NV) {
+        const uint32_t col = VEC * (ptau + (uint32_t)JC * TPP);
+        bcold_levels<W, LC, VEC, JC * VEC * (1 << LC), 0, RR>(v, __brev(col >> BB) >> (32 - (RW - BB)), tw, c);
+        bcold_all<W, LC, RW, VEC, TPP, JC + 1, NV, RR>(v, ptau, tw, c);
     }
 }
 
-template <typename W, int L, int LROW = L, int BLK = BLOCK>
+// A row group of the column/row kernels: TPP threads hold one sequence pair
+// of 2^LROW elements, as RC rows of 2^RW.  FULL (whole sequences): block
+// form, rows padded for vector access, the first N / 8 pairs of the table in
+// shared memory, VEC adjacent columns per thread access.  Otherwise (rows of
+// the split path's row-twiddle form): the complete transform, twiddles from
+// the plan's table.
+template <typename W, int LROW, bool FULL, int BLK = BLOCK>
 struct CRShape {
     static constexpr int RW = Arith<W>::RB + 5;
     static constexpr int LC = LROW - RW;                    // column bits inside one row
     static constexpr int RC = 1 << LC;
-    using GR = Geo<W, RW>;
+    static constexpr int ROWP = FULL ? BGeo<W, RW>::ROWP : Geo<W, RW>::ROWP;
     static constexpr int TPP = 32 * RC;                     // threads per row
     static constexpr int PPC = BLK / TPP;                   // rows per block
     static_assert(PPC >= 1, "a row needs more threads than the block has");
     static constexpr int CPT = (1 << RW) / TPP;             // columns per thread
-    // shared twiddles: the whole table (whole sequences) or only the entries
-    // below 2^(LROW-1) that the inverse levels inside a row read (split rows)
-    static constexpr int TWL = (L == LROW) ? L : 0;         // split rows read the plan's table
-    static constexpr size_t smem = TwBytes<W, TWL>::v + (size_t)PPC * RC * 2 * GR::ROWP * sizeof(W);
+    static constexpr int VEC = CPT < (int)(16 / sizeof(W)) ? CPT : (int)(16 / sizeof(W));
+    static constexpr int TWL = LROW - BB;                   // TwBytes: 2^(TWL - 1) pairs
+    static constexpr size_t tw_bytes = FULL ? TwBytes<W, TWL>::v : 0;
+    static constexpr size_t rows_bytes = (size_t)PPC * RC * 2 * ROWP * sizeof(W);
+    static constexpr bool STAGE = FULL && sizeof(W) == 4;   // the next pair staged by asynchronous copies
+    static constexpr size_t smem = tw_bytes + rows_bytes + (STAGE ? (size_t)PPC * (sizeof(W) << LROW) : 0);   // and its g
 };
 
-// Column/row fused convolution.  L == LROW: whole sequences (f, g, h or the
-// descriptor list; output canonical at <-x>_N).  L > LROW: one row of 2^LROW
-// elements of the split path per row group, inputs F~, G~ and output H~ in
-// the wave's scratch; the forward node twiddles of such a row depend on the
-// row and are read from the plan's table, the inverse ones do not and are
-// read from shared memory.
+// One row of 2^RW words by a warp's asynchronous copies, to a padded or a
+// plain row in shared memory; 16 bytes each where source and layout allow.
+template <typename W, int RW, bool PADDED>
+__device__ __forceinline__ void stage_row(const W *src, W *dst, uint32_t lane)
+{
+    using GR = BGeo<W, RW>;
+    constexpr uint32_t Q = (uint32_t)(16 / sizeof(W));
+    if ((GR::VX || !PADDED) && ((uintptr_t)src & 15u) == 0) {
+#pragma unroll
+        for (uint32_t i = 0; i < (1u << RW) / (32 * Q); ++i) {
+            const uint32_t e = (lane + 32u * i) * Q;
+            cp_async<16>(dst + (PADDED ? GR::pad(e) : e), src + e);
+        }
+    } else {
+#pragma unroll 8
+        for (uint32_t i = 0; i < (1u << RW) / 32; ++i) {
+            const uint32_t e = lane + 32u * i;
+            cp_async<sizeof(W)>(dst + (PADDED ? GR::pad(e) : e), src + e);
+        }
+    }
+}
+
+// A thread's columns (VEC adjacent ones at VEC ptau + j VEC TPP, 2^LC
+// elements each) from rows in shared memory.
+template <typename W, int RW, int LC, int VEC, int TPP, bool PADDED, int R>
+__device__ __forceinline__ void cols_from_rows(const W *S, uint32_t stride, uint32_t ptau, W (&v)[R])
+{
+    using GR = BGeo<W, RW>;
+#pragma unroll
+    for (int j = 0; j < (R >> LC) / VEC; ++j)
+#pragma unroll
+        for (int k = 0; k < (1 << LC); ++k) {
+            const uint32_t c = VEC * (ptau + (uint32_t)j * TPP);
+            W t[VEC];
+            ld_vec<W, VEC>(S + (size_t)k * stride + (PADDED ? GR::pad(c) : c), t, GR::VX || !PADDED);
+#pragma unroll
+            for (int e = 0; e < VEC; ++e) v[((j * VEC + e) << LC) + k] = t[e];
+        }
+}
+
+// Column/row fused convolution of whole sequences (f, g, h or the descriptor
+// list), by blocks (ntt_block.cuh).
 // Rows [base + row group, end) by steps of stride; end is a.nrows unless ITEM.
-// OUT 0: canonical at <-x>_N (a whole convolution); OUT 1: lazy residues in
-// natural order (a row of a convolution's split path, after the twist).
-template <typename W, int L, int LROW, int SRC, bool ITEM = false, int OUT = 0, class X = NoExact, int BLK = BLOCK>
+// OUT 0: canonical, at block_out(x) (a whole convolution); OUT 1: lazy
+// residues of a row of a convolution's split path, after the twist: element
+// 4 t' + r goes to <4 t' - r>, where the transposed column pass reads it (its
+// output stage reverses the whole index); the factor 2^(B + BB) / N is in
+// the twist's diagonal.
+template <typename W, int L, int SRC, bool ITEM = false, int OUT = 0, class X = NoExact, int BLK = BLOCK>
 __device__ __forceinline__ void conv_cr_body(const RowArgs<W> &a, long long base, long long stride, long long end = 0,
                                              const ExactArgs *xa = nullptr)
 {
-    using SH = CRShape<W, L, LROW, BLK>;
-    using GR = typename SH::GR;
-    constexpr int RW = SH::RW, LC = SH::LC, RC = SH::RC, TPP = SH::TPP, PPC = SH::PPC, CPT = SH::CPT;
+    using SH = CRShape<W, L, true, BLK>;
+    constexpr int RW = SH::RW, LC = SH::LC, RC = SH::RC, TPP = SH::TPP, PPC = SH::PPC, CPT = SH::CPT, VEC = SH::VEC;
+    using GR = BGeo<W, RW>;
     constexpr int R = GR::R;
     static_assert(LC >= 1 && CPT * RC == R, "column/row split");
-    constexpr bool FULL = (L == LROW);
-    constexpr int FTW = FULL ? TW_SMEM : TW_GLOBAL;         // forward twiddle source
     constexpr uint32_t N = 1u << L;
     constexpr int last = GR::NPASS - 1;
+    constexpr bool STAGE = SH::STAGE && !X::IN64;
+    constexpr uint32_t INB = X::IN64 ? 8u : (uint32_t)sizeof(W);     // bytes per input element
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int pid = threadIdx.x / TPP;
     const uint32_t ptau = threadIdx.x % TPP;
     const int wr = (int)(ptau >> 5);
     const uint32_t lane = ptau & 31u;
     W *stw = reinterpret_cast<W *>(smem_raw);
-    W *P = reinterpret_cast<W *>(smem_raw + TwBytes<W, SH::TWL>::v) + (size_t)pid * RC * 2 * GR::ROWP;
+    W *P = reinterpret_cast<W *>(smem_raw + SH::tw_bytes) + (size_t)pid * RC * 2 * GR::ROWP;
     W *Srow = P + (size_t)wr * 2 * GR::ROWP;                // this warp's g slice (also H); f slice follows
-    const W *ftw = FULL ? stw : a.tw;
-    const uint32_t b0 = GR::base(0, lane);
-    constexpr int lo0 = GR::lo(0);
-    if constexpr (FULL) {
-        stage_twiddles<W>(a.tw, stw, TwBytes<W, SH::TWL>::pairs);
-        __syncthreads();
-    }
+    stage_twiddles<W>(a.tw, stw, TwBytes<W, SH::TWL>::pairs);
+    __syncthreads();
 
     // The row groups of a block synchronise block-wide and step through the
     // rows in rounds together (a group whose row of the round is past the
@@ -387,142 +439,249 @@ __device__ __forceinline__ void conv_cr_body(const RowArgs<W> &a, long long base
     // the same time: measured 9% (2^11) and 15% (2^12) faster than a
     // barrier per group, whose groups drift apart across the unrolled code.
     auto psync = [&]() { __syncthreads(); };
-    auto ptrs = [&](long long rho, const W *&fp, const W *&gp, W *&hp, uint32_t &rowoff) {
-        if constexpr (FULL) {
-            const long long pair = a.pair0 + rho;
-            if constexpr (SRC == 1) {
-                const DevDesc<W> d = a.descs[pair];
-                fp = d.f; gp = d.g; hp = d.h;
-            } else {
-                fp = seq_base<X>(a.f, pair, N); gp = seq_base<X>(a.g, pair, N);
-                hp = X::GARNER ? nullptr : a.h + (size_t)pair * N;
-            }
-            rowoff = 0;
+    auto ptrs = [&](long long rho, const W *&fp, const W *&gp, W *&hp) {
+        const long long pair = a.pair0 + rho;
+        if constexpr (SRC == 1) {
+            const DevDesc<W> d = a.descs[pair];
+            fp = d.f; gp = d.g; hp = d.h;
         } else {
-            const long long pw = rho >> (L - LROW);
-            const uint32_t row = (uint32_t)rho & ((1u << (L - LROW)) - 1u);
-            const size_t off = (size_t)pw * N + ((size_t)row << LROW);
-            fp = a.f + off; gp = a.g + off; hp = a.h + off;
-            rowoff = row << LROW;
+            fp = seq_base<X>(a.f, pair, N); gp = seq_base<X>(a.g, pair, N);
+            hp = X::GARNER ? nullptr : a.h + (size_t)pair * N;
         }
     };
-    // v[1] carries this row's f, loaded during the previous row's inverse
-    // phases (the registers are free after the pointwise product); g is
-    // loaded into v[0] while f's column levels run.  (Staging g in the idle
-    // g slices with cp.async instead was measured slower: the extra shared
-    // memory traffic costs more than the latency it hides.)
-    auto load_cols = [&](const W *src, W (&dst)[R]) {
+    // A thread's columns: VEC adjacent ones at VEC ptau + j VEC TPP; column c
+    // holds the elements c + k 2^RW, k < RC, in registers (j VEC + e) RC + k.
+    auto col_of = [&](int j) { return VEC * (ptau + (uint32_t)j * TPP); };
+    auto load_cols = [&](const W *src, W (&dst)[R]) {       // from global memory (X::IN64: reduced on the way)
+        auto all = [&](bool wide) {
 #pragma unroll
-        for (int j = 0; j < CPT; ++j)
+            for (int j = 0; j < CPT / VEC; ++j)
 #pragma unroll
-            for (int k = 0; k < RC; ++k) dst[j * RC + k] = ld_elem<X>(src, ptau + (uint32_t)j * TPP + ((uint32_t)k << RW), xa);
+                for (int k = 0; k < RC; ++k) {
+                    const uint32_t x = col_of(j) + ((uint32_t)k << RW);
+                    W t[VEC];
+                    if constexpr (X::IN64) {
+#pragma unroll
+                        for (int e = 0; e < VEC; ++e) t[e] = ld_elem<X>(src, x + e, xa);
+                    } else {
+                        ld_vec<W, VEC>(src + x, t, wide);
+                    }
+#pragma unroll
+                    for (int e = 0; e < VEC; ++e) dst[(j * VEC + e) * RC + k] = t[e];
+                }
+        };
+        if (!X::IN64 && VEC > 1 && ((uintptr_t)src & (VEC * sizeof(W) - 1)) == 0) all(true);
+        else all(false);
     };
-    constexpr uint32_t INB = X::IN64 ? 8u : (uint32_t)sizeof(W);     // bytes per input element
+    auto store_cols = [&](const W (&v)[R], W *S) {          // into the rows' slices
+#pragma unroll
+        for (int j = 0; j < CPT / VEC; ++j)
+#pragma unroll
+            for (int k = 0; k < RC; ++k) {
+                W t[VEC];
+#pragma unroll
+                for (int e = 0; e < VEC; ++e) t[e] = v[(j * VEC + e) * RC + k];
+                st_vec<W, VEC>(S + (size_t)k * 2 * GR::ROWP + GR::pad(col_of(j)), t, GR::VX);
+            }
+    };
+    // STAGE (32-bit words): the next pair arrives by asynchronous copies
+    // while this one is convolved: each warp brings its own row of f into its
+    // f slice (free after the block products) and of g into the staging rows
+    // G (read before the first barrier); the wait before the second barrier
+    // makes both visible to the columns of the next round.  No register
+    // holds loaded words across the inverse, and no load waits on L2:
+    // measured on GB300, 4096 x 2^14 412 -> 394 us at equal clocks (without
+    // any global load: 369), 8192 x 2^13 392 -> 376, 2^12 1.5%, 2^11 equal.
+    // 64-bit words, whose padded rows take 8-byte copies only, lose by it
+    // (301 x 2^13: 59.4 -> 61.5 us); there the next f is loaded into registers
+    // after the block products, and g while f's columns are transformed.
+    W *G = reinterpret_cast<W *>(smem_raw + SH::tw_bytes + SH::rows_bytes) + ((size_t)pid << L);
+    auto stage_f = [&](const W *f) { stage_row<W, RW, true>(f + ((size_t)wr << RW), Srow + GR::ROWP, lane); };
+    auto stage_g = [&](const W *g) { stage_row<W, RW, false>(g + ((size_t)wr << RW), G + ((size_t)wr << RW), lane); };
     const long long lim = ITEM ? end : a.nrows;
     W v[2][R];
     const W *fp = nullptr, *gp = nullptr;
     W *hp = nullptr;
-    uint32_t rowoff = 0;
-    // (split rows keep no prefetched registers across their inverse: it reads
-    // its twiddles from global memory and needs the registers itself)
-    constexpr bool PREF = FULL;
-    if (PREF && base + pid < lim) {
-        ptrs(base + pid, fp, gp, hp, rowoff);
-        load_cols(fp, v[1]);
+    if (base + pid < lim) {
+        ptrs(base + pid, fp, gp, hp);
+        if constexpr (STAGE) {
+            stage_f(fp);
+            stage_g(gp);
+        } else {
+            load_cols(fp, v[1]);
+        }
+    }
+    if constexpr (STAGE) {
+        cp_async_wait();
+        psync();
     }
     for (long long round = base; round < lim; round += stride) {
         const long long rho = round + pid;
         const bool live = PPC == 1 || rho < lim;            // this group's row of the round exists
-        if (!PREF && live) {
-            ptrs(rho, fp, gp, hp, rowoff);
-            load_cols(fp, v[1]);
-        }
+        const bool more = rho + stride < lim;
         W *const hcur = hp;
-        const uint32_t rcur = live ? rowoff : 0u;
-        const W *gcur = gp;
-        if (ptau == 0 && rho + stride < lim) {
-            const W *fn, *gn;
-            W *hn;
-            uint32_t ro;
-            ptrs(rho + stride, fn, gn, hn, ro);
-            prefetch_l2(fn, (1u << LROW) * INB);
-            prefetch_l2(gn, (1u << LROW) * INB);
+        if constexpr (!STAGE) {
+            if (ptau == 0 && more) {
+                const W *fn, *gn;
+                W *hn;
+                ptrs(rho + stride, fn, gn, hn);
+                prefetch_l2(fn, N * INB);
+                prefetch_l2(gn, N * INB);
+            }
+            if (live) load_cols(gp, v[0]);
         }
-        // forward, column phase: columns c = ptau + j TPP, elements x = c + k 2^RW.
-        // No barrier before the column stores: the f slices were last read in
-        // the previous row's row phase, before the last barrier, and in the g
-        // slices every thread writes only the positions of its own columns,
-        // which it alone read in the previous row's inverse column phase.
-        // (Measured on GB300 at 4096 x 2^14: moving the barrier that stood
-        // before both stores to after f's made the kernel 2.9% faster,
-        // removing it 0.8% more.)
-        if (live) load_cols(gcur, v[0]);
-        colf_all<W, LC, 0, CPT, L - LROW, FTW, R>(v[1], rcur >> RW, ftw, a.c);
-#pragma unroll
-        for (int j = 0; j < CPT; ++j)
-#pragma unroll
-            for (int k = 0; k < RC; ++k) {
-                const uint32_t y = ptau + (uint32_t)j * TPP;
-                P[(size_t)k * 2 * GR::ROWP + GR::ROWP + GR::pad(y)] = v[1][j * RC + k];   // f
-            }
-        colf_all<W, LC, 0, CPT, L - LROW, FTW, R>(v[0], rcur >> RW, ftw, a.c);
-#pragma unroll
-        for (int j = 0; j < CPT; ++j)
-#pragma unroll
-            for (int k = 0; k < RC; ++k) {
-                const uint32_t y = ptau + (uint32_t)j * TPP;
-                P[(size_t)k * 2 * GR::ROWP + GR::pad(y)] = v[0][j * RC + k];              // g
-            }
+        // forward, column phase.
+        // No barrier before the column stores: in the slices every thread
+        // writes only the positions of its own columns, which it alone read
+        // here (f) or in the previous row's inverse column phase (g).
+        if constexpr (STAGE) cols_from_rows<W, RW, LC, VEC, TPP, true>(P + GR::ROWP, 2 * GR::ROWP, ptau, v[1]);
+        colf_all<W, LC, 0, CPT, 0, TW_SMEM, R>(v[1], 0u, stw, a.c);
+        store_cols(v[1], P + GR::ROWP);
+        if constexpr (STAGE) cols_from_rows<W, RW, LC, VEC, TPP, false>(G, 1u << RW, ptau, v[0]);
+        colf_all<W, LC, 0, CPT, 0, TW_SMEM, R>(v[0], 0u, stw, a.c);
+        store_cols(v[0], P);
         psync();
-        // forward, row phase (warp wr owns row wr of this row group)
+        if (more) {
+            ptrs(rho + stride, fp, gp, hp);
+            if constexpr (STAGE) stage_g(gp);
+        }
+        // row phase (warp wr owns row wr of this row group): forward, block
+        // products, inverse
+        bload<W, RW, 0>(v[0], Srow, lane);
+        bload<W, RW, 0>(v[1], Srow + GR::ROWP, lane);
+        bfwd_all<W, L, RW, 0, false>(v, (uint32_t)wr << RW, lane, Srow, 0, stw, a.c);
+        block_products<W, R>(v, ((uint32_t)wr << RW) + GR::base(last, lane), stw, a.c);
+        if (more) {
+            if constexpr (STAGE) {
+                __syncwarp();
+                stage_f(fp);
+            } else {
+                load_cols(fp, v[1]);
+            }
+        }
+        bdit_all<W, RW, last>(v[0], lane, Srow, 0, stw, a.c);
+        bstore<W, RW, 0>(v[0], Srow, lane);
+        if constexpr (STAGE) cp_async_wait();
+        psync();
+        // inverse, column phase
+        cols_from_rows<W, RW, LC, VEC, TPP, true>(P, 2 * GR::ROWP, ptau, v[0]);
+        bcold_all<W, LC, RW, VEC, TPP, 0, CPT / VEC, R>(v[0], ptau, stw, a.c);
+        if (!live) continue;                                // (no barrier follows in this round)
+        const bool wide = ((uintptr_t)hcur & (VEC * sizeof(W) - 1)) == 0;
+#pragma unroll
+        for (int j = 0; j < CPT / VEC; ++j)
+#pragma unroll
+            for (int k = 0; k < RC; ++k) {
+                const uint32_t x = col_of(j) + ((uint32_t)k << RW);
+                W t[VEC];
+#pragma unroll
+                for (int e = 0; e < VEC; ++e) t[e] = v[0][(j * VEC + e) * RC + k];
+                if constexpr (OUT == 1) {
+#pragma unroll
+                    for (int e = 0; e < VEC; ++e) hcur[(x + e - 2 * ((x + e) & 3u)) & (N - 1u)] = t[e];
+                } else {
+#pragma unroll
+                    for (int e = 0; e < VEC; ++e) t[e] = canon<W>(t[e], a.c.cB, a.c.cBp, a.c.m);
+                    if constexpr (X::GARNER) {
+#pragma unroll
+                        for (int e = 0; e < VEC; ++e) st_out<X>(hcur, a.pair0 + rho, N, block_out<L>(x + e), t[e], xa);
+                    } else {
+                        st_vec<W, VEC>(hcur + block_out<L>(x), t, wide);
+                    }
+                }
+            }
+    }
+}
+
+template <typename W, int L, int SRC, int OUT = 0, int BLK = BLOCK>
+__global__ void __launch_bounds__(BLK, BLOCK / BLK) k_conv_cr(const __grid_constant__ RowArgs<W> a)
+{
+    constexpr int PPC = CRShape<W, L, true, BLK>::PPC;
+    conv_cr_body<W, L, SRC, false, OUT, NoExact, BLK>(a, (long long)blockIdx.x * PPC, (long long)gridDim.x * PPC);
+}
+
+// Rows of the split path's row-twiddle form: one row of 2^LROW elements of
+// the length-2^L tree per row group, inputs F~, G~ and output H~ (lazy
+// residues, natural order) in the wave's scratch.  The node twiddles depend
+// on the row and are read from the plan's table; the inverse is the
+// transposed tree, whose twiddles (like the forward ones) are contiguous
+// runs of it.  The complete transform with a pointwise product.
+template <typename W, int L, int LROW>
+__global__ void __launch_bounds__(BLOCK, 1) k_conv_rows(const __grid_constant__ RowArgs<W> a)
+{
+    using SH = CRShape<W, LROW, false>;
+    using GR = Geo<W, SH::RW>;
+    constexpr int RW = SH::RW, LC = SH::LC, RC = SH::RC, TPP = SH::TPP, PPC = SH::PPC, CPT = SH::CPT;
+    constexpr int R = GR::R;
+    static_assert(PPC == 1 && LC >= 1 && CPT * RC == R, "one row per block");
+    constexpr uint32_t N = 1u << L;
+    constexpr int last = GR::NPASS - 1;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const uint32_t ptau = threadIdx.x;
+    const int wr = (int)(ptau >> 5);
+    const uint32_t lane = ptau & 31u;
+    W *P = reinterpret_cast<W *>(smem_raw);
+    W *Srow = P + (size_t)wr * 2 * GR::ROWP;                // this warp's g slice (also H); f slice follows
+    const uint32_t b0 = GR::base(0, lane);
+    constexpr int lo0 = GR::lo(0);
+    for (long long rho = blockIdx.x; rho < a.nrows; rho += gridDim.x) {
+        const uint32_t row = (uint32_t)rho & ((1u << (L - LROW)) - 1u);
+        const size_t off = (size_t)(rho >> (L - LROW)) * N + ((size_t)row << LROW);
+        const W *fp = a.f + off, *gp = a.g + off;
+        W *hp = a.h + off;
+        const uint32_t rowoff = row << LROW;
+        W v[2][R];
+        auto load_cols = [&](const W *src, W (&dst)[R]) {
+#pragma unroll
+            for (int j = 0; j < CPT; ++j)
+#pragma unroll
+                for (int k = 0; k < RC; ++k) dst[j * RC + k] = src[ptau + (uint32_t)j * TPP + ((uint32_t)k << RW)];
+        };
+        auto store_cols = [&](const W (&s)[R], W *S) {
+#pragma unroll
+            for (int j = 0; j < CPT; ++j)
+#pragma unroll
+                for (int k = 0; k < RC; ++k) S[(size_t)k * 2 * GR::ROWP + GR::pad(ptau + (uint32_t)j * TPP)] = s[j * RC + k];
+        };
+        load_cols(fp, v[1]);
+        if (ptau == 0 && rho + gridDim.x < a.nrows) {
+            const long long nx = rho + gridDim.x;
+            const size_t no = (size_t)(nx >> (L - LROW)) * N + ((size_t)((uint32_t)nx & ((1u << (L - LROW)) - 1u)) << LROW);
+            prefetch_l2(a.f + no, (uint32_t)(sizeof(W) << LROW));
+            prefetch_l2(a.g + no, (uint32_t)(sizeof(W) << LROW));
+        }
+        load_cols(gp, v[0]);
+        // (no barrier before the column stores: see conv_cr_body)
+        colf_all<W, LC, 0, CPT, L - LROW, TW_GLOBAL, R>(v[1], rowoff >> RW, a.tw, a.c);
+        store_cols(v[1], P + GR::ROWP);
+        colf_all<W, LC, 0, CPT, L - LROW, TW_GLOBAL, R>(v[0], rowoff >> RW, a.tw, a.c);
+        store_cols(v[0], P);
+        __syncthreads();
 #pragma unroll
         for (int k = 0; k < R; ++k) {
             const uint32_t y = b0 + ((uint32_t)k << lo0);
             v[0][k] = Srow[GR::pad(y)];
             v[1][k] = Srow[GR::ROWP + GR::pad(y)];
         }
-        fwd_all<W, L, RW, 0, 2, FTW>(v, rcur + ((uint32_t)wr << RW), lane, Srow, 0, ftw, a.c);
+        fwd_all<W, L, RW, 0, 2, TW_GLOBAL>(v, rowoff + ((uint32_t)wr << RW), lane, Srow, 0, a.tw, a.c);
 #pragma unroll
         for (int k = 0; k < R; ++k) v[0][k] = pointwise(v[1][k], v[0][k], a.c);
-        if (PREF && rho + stride < lim) {
-            ptrs(rho + stride, fp, gp, hp, rowoff);
-            load_cols(fp, v[1]);                            // next row's f
-        }
-        // inverse, row phase: decimation in time for whole sequences; for a
-        // row of the split path the transposed tree, whose twiddles (like the
-        // forward ones) are contiguous runs of the plan's table
-        if constexpr (FULL) dit_all<W, RW, last, TW_SMEM>(v[0], (uint32_t)wr << RW, lane, Srow, 0, stw, a.c);
-        else inv_all<W, L, RW, last, TW_GLOBAL>(v[0], rcur + ((uint32_t)wr << RW), lane, Srow, 0, a.tw, a.c);
+        inv_all<W, L, RW, last, TW_GLOBAL>(v[0], rowoff + ((uint32_t)wr << RW), lane, Srow, 0, a.tw, a.c);
 #pragma unroll
         for (int k = 0; k < R; ++k) Srow[GR::pad(b0 + ((uint32_t)k << lo0))] = v[0][k];
-        psync();
-        // inverse, column phase
+        __syncthreads();
 #pragma unroll
         for (int j = 0; j < CPT; ++j) {
             const uint32_t col = ptau + (uint32_t)j * TPP;
 #pragma unroll
             for (int k = 0; k < RC; ++k) v[0][j * RC + k] = P[(size_t)k * 2 * GR::ROWP + GR::pad(col)];
         }
-        if constexpr (FULL) cold_all<W, LC, RW, 0, CPT, TPP, TW_SMEM, R>(v[0], ptau, stw, a.c);
-        else colg_all<W, LC, 0, CPT, L - LROW, TW_GLOBAL, R>(v[0], rcur >> RW, a.tw, a.c);
-        if (!live) continue;                                // (no barrier follows in this round)
+        colg_all<W, LC, 0, CPT, L - LROW, TW_GLOBAL, R>(v[0], rowoff >> RW, a.tw, a.c);
 #pragma unroll
         for (int j = 0; j < CPT; ++j)
 #pragma unroll
-            for (int k = 0; k < RC; ++k) {
-                const uint32_t x = ptau + (uint32_t)j * TPP + ((uint32_t)k << RW);
-                if constexpr (FULL && OUT == 0)
-                    st_out<X>(hcur, a.pair0 + rho, N, (N - x) & (N - 1u), canon<W>(v[0][j * RC + k], (W)1, a.c.onep, a.c.m), xa);
-                else hcur[x] = v[0][j * RC + k];
-            }
+            for (int k = 0; k < RC; ++k) hp[ptau + (uint32_t)j * TPP + ((uint32_t)k << RW)] = v[0][j * RC + k];
     }
-}
-
-template <typename W, int L, int LROW, int SRC, int OUT = 0, int BLK = BLOCK>
-__global__ void __launch_bounds__(BLK, BLOCK / BLK) k_conv_cr(const __grid_constant__ RowArgs<W> a)
-{
-    constexpr int PPC = CRShape<W, L, LROW, BLK>::PPC;
-    conv_cr_body<W, L, LROW, SRC, false, OUT, NoExact, BLK>(a, (long long)blockIdx.x * PPC, (long long)gridDim.x * PPC);
 }
 
 // The exact convolution's fused launches (whole sequences, contiguous):
@@ -534,11 +693,11 @@ __global__ void __launch_bounds__(BLOCK, 1) k_conv_exact(const __grid_constant__
 {
     constexpr int RW = Arith<W>::RB + 5;
     if constexpr (L <= RW) {
-        constexpr int GPC = RowShape<W, L, L>::GPC;
+        constexpr int GPC = FusedShape<W, L>::GPC;
         conv_fused_body<W, L, 0, X>(a, (long long)blockIdx.x * GPC, (long long)gridDim.x * GPC, &e);
     } else {
-        constexpr int PPC = CRShape<W, L, L>::PPC;
-        conv_cr_body<W, L, L, 0, false, 0, X>(a, (long long)blockIdx.x * PPC, (long long)gridDim.x * PPC, 0, &e);
+        constexpr int PPC = CRShape<W, L, true>::PPC;
+        conv_cr_body<W, L, 0, false, 0, X>(a, (long long)blockIdx.x * PPC, (long long)gridDim.x * PPC, 0, &e);
     }
 }
 
@@ -578,9 +737,9 @@ __device__ __forceinline__ void persist_item(const PersistArgs<W> &a, const Work
     if constexpr (L <= RW) {
         RowArgs<W> ra = a.cls[L];
         ra.nrows = w.first + w.count;
-        conv_fused_body<W, L, 1>(ra, w.first, RowShape<W, L, L>::GPC);
+        conv_fused_body<W, L, 1>(ra, w.first, FusedShape<W, L>::GPC);
     }
-    else conv_cr_body<W, L, L, 1, true>(a.cls[L], w.first, CRShape<W, L, L>::PPC, w.first + w.count);
+    else conv_cr_body<W, L, 1, true>(a.cls[L], w.first, CRShape<W, L, true>::PPC, w.first + w.count);
 }
 
 template <typename W, int L, int HI>
@@ -1078,7 +1237,9 @@ __global__ void __launch_bounds__(BLOCK, 1) k_rows_uni(const __grid_constant__ R
 }
 
 // Bit-reversal gather of a split-path spectrum: y[u] = X(u) from the tree
-// order (X(brv(x)) at x); INV applies <-u>_N and N^-1.  Canonical outputs.
+// order (X(brv(x)) at x); INV applies <-u>_N.  The factor c.ninv is the
+// caller's: N^-1 for the inverse, and what undoes the scale of the twist's
+// diagonal.  Canonical outputs.
 template <typename W, int L, bool INV>
 __global__ void k_bitrev_out(const W *__restrict__ src, W *__restrict__ dst, long long batch, ModC<W> c)
 {
@@ -1089,9 +1250,7 @@ __global__ void k_bitrev_out(const W *__restrict__ src, W *__restrict__ dst, lon
     const uint32_t t = (uint32_t)idx & (N - 1u);
     const uint32_t u = INV ? ((N - t) & (N - 1u)) : t;
     const uint32_t x = __brev(u) >> (32 - L);
-    const W scale = INV ? c.ninv : (W)1;
-    const W scalep = INV ? c.ninvp : c.onep;
-    dst[idx] = csub<W>(shoup<W>(src[(size_t)b * N + x], scale, scalep, c.m), c.m);
+    dst[idx] = csub<W>(shoup<W>(src[(size_t)b * N + x], c.ninv, c.ninvp, c.m), c.m);
 }
 
 // The same gather, tiled (L >= 10): write an index as (h, m, l) with h and
@@ -1116,8 +1275,6 @@ __global__ void __launch_bounds__(256) k_bitrev_tiled(const W *__restrict__ src,
     const uint32_t lane = threadIdx.x & 31u, wid = threadIdx.x >> 5;
     const W *s = src + (size_t)b * N;
     W *d = dst + (size_t)b * N;
-    const W scale = INV ? c.ninv : (W)1;
-    const W scalep = INV ? c.ninvp : c.onep;
     // source runs: x = (sh, mb, sl), sh = brv(ul) fixed per run, sl = lane
 #pragma unroll
     for (int r = 0; r < 4; ++r) {
@@ -1131,7 +1288,7 @@ __global__ void __launch_bounds__(256) k_bitrev_tiled(const W *__restrict__ src,
         const uint32_t uh = wid * 4 + r;
         const uint32_t u = (uh << (L - 5)) | (m << 5) | lane;
         const W v = tile[__brev(lane) >> 27][__brev(uh) >> 27];
-        d[INV ? ((N - u) & (N - 1u)) : u] = csub<W>(shoup<W>(v, scale, scalep, c.m), c.m);
+        d[INV ? ((N - u) & (N - 1u)) : u] = csub<W>(shoup<W>(v, c.ninv, c.ninvp, c.m), c.m);
     }
 }
 
