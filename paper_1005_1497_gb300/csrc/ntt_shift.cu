@@ -17,12 +17,26 @@
 // SHOUP mode is the same kernel with every twiddle applied as a Shoup
 // product modulo m (the multiply form of the main path), for comparison.
 //
-// Layout: P = min(32, N) lanes per pair, E = N / P (1 or 2) elements per
-// lane, element x = q + P k (q = lane in the group).  Butterflies at a
-// distance below P exchange values with __shfl_xor_sync; at distance P
-// (N = 64) they are inside the lane.  Forward: the node tree of the main
-// path (node i = x >> (L - d), twiddle w^brv(i)); inverse: its transpose
-// (Gentleman-Sande butterflies, same twiddles), output at <-x>_N.
+// Layout.  E = min(8, N) elements per thread, T = N / E threads per pair.
+// Pass 1: a thread holds x = q + T k (k < E, q its place among the T), so
+// the three top levels act inside it and their shift amounts are compile-time constants.
+// Pass 2 (N > 8): after an exchange through the warp's shared memory it
+// holds x = E q + k, and the remaining levels' amounts are one exponent of q
+// and constants.  Forward: the node tree of the main path (node i = x >> (L -
+// d), twiddle w^brv(i)); inverse: its transpose, output at <-x>_N.  Every
+// pair's words move as whole 32-byte sectors.
+//
+// SHIFT mode keeps values lazily, as signed words (64 bits for F_5, 32 for
+// F_4): a twiddle product leaves lo - hi without a fix-up and sums are never
+// reduced.  |x| < 2^36 after the forward levels and < 2^40 after the inverse ones
+// for F_5 (inputs < 2^23, each level adds at most 2^32 + half the bound),
+// < 2^21 and < 2^24 for F_4 (K = 16).
+//
+// What bounds it: integer instructions (five for a twiddle product, four for
+// a butterfly's sums; the schedulers issue in 77% of cycles, the ALU pipe is
+// 76% busy).  Measured on GB300 at 1000003 x 64, m = 641: 252 us, 3.0 TB/s
+// (0.45 of the copy rate); one or two elements per lane, with shuffles at
+// every level and each sum reduced to [0, F_t], took 1772 us.
 #include <cuda_runtime.h>
 
 #include <cstring>
@@ -47,49 +61,9 @@ struct ShiftArgs {
     uint32_t z[32];
     uint32_t zp[32];
     uint32_t ninv, ninvp;    // N^-1 mod m, Shoup quotient (SHOUP mode)
+    uint32_t onep32;         // floor(2^32 / m)
+    uint32_t big;            // the largest multiple of m below 2^31
 };
-
-// ---- arithmetic modulo F_t = 2^K + 1, K = 2^t, values in [0, 2^K] ----
-template <int K>
-__device__ __forceinline__ uint64_t f_reduce(uint64_t y)     // y < 2^(2K): y = hi 2^K + lo = lo - hi
-{
-    constexpr uint64_t F = (1ull << K) + 1;
-    const uint64_t lo = y & ((1ull << K) - 1), hi = y >> K;
-    return lo >= hi ? lo - hi : lo + F - hi;
-}
-template <int K>
-__device__ __forceinline__ uint64_t f_add(uint64_t a, uint64_t b)
-{
-    constexpr uint64_t F = (1ull << K) + 1;
-    const uint64_t s = a + b;
-    return s >= F ? s - F : s;
-}
-template <int K>
-__device__ __forceinline__ uint64_t f_sub(uint64_t a, uint64_t b)
-{
-    constexpr uint64_t F = (1ull << K) + 1;
-    return a >= b ? a - b : a + F - b;
-}
-template <int K>
-__device__ __forceinline__ uint64_t f_shl(uint64_t b, uint32_t e)  // b 2^e, e < K, b <= 2^K: b << e < 2^(2K)
-{
-    return f_reduce<K>(b << e);
-}
-template <int K>
-__device__ __forceinline__ uint64_t f_mul(uint64_t a, uint64_t b)  // general product (pointwise only)
-{
-    constexpr uint64_t F = (1ull << K) + 1;
-    if (a == (1ull << K)) return b == 0 ? 0 : F - b;               // 2^K = -1
-    if (b == (1ull << K)) return a == 0 ? 0 : F - a;
-    return f_reduce<K>(a * b);                                      // a, b < 2^K: a b < 2^(2K)
-}
-
-// ---- arithmetic modulo m (SHOUP mode), canonical values ----
-__device__ __forceinline__ uint32_t m_shoup(uint32_t b, uint32_t z, uint32_t zp, uint32_t m)
-{
-    uint32_t r = b * z - __umulhi(b, zp) * m;
-    return r >= m ? r - m : r;
-}
 
 // Exponent of the twiddle of node i at length 2^L: w = 2^(2K/N), z_i = w^brv_{L-1}(i).
 template <int K, int L>
@@ -98,115 +72,210 @@ __device__ __forceinline__ uint32_t tw_exp(uint32_t i)
     return (2u * K >> L) * (__brev(i) >> (32 - (L - 1 > 0 ? L - 1 : 1))) * (L > 1 ? 1u : 0u);
 }
 
-template <int K, int L, bool SHIFT>
-struct Ops {
-    using V = uint64_t;
-    __device__ static V tw(V b, uint32_t node, const ShiftArgs &a)
+// Values, twiddles and reductions of the two modes.
+//   Tw: a node's twiddle (an exponent e < K, or a factor and its quotient);
+//   mul(b, t): b times it; lift(v): a word in [0, 2^32) equal to v modulo m;
+//   point(F, G): F G N^-1; out(v): the canonical residue modulo m.
+// Inverse level j (0 the first): sub(x, y, j) is x - y.
+template <int K, int L, bool SHIFT> struct Ops;
+
+// ---- modulo F_5 = 2^32 + 1, signed 64-bit words ----
+template <int L> struct Ops<32, L, true> {
+    using V = int64_t;
+    using Tw = uint32_t;
+    __device__ __forceinline__ static V load(uint32_t x) { return (V)x; }
+    __device__ __forceinline__ static Tw node(uint32_t i, const ShiftArgs &) { return tw_exp<32, L>(i); }
+    // b 2^e = B1 2^32 + B0 2^e, B0 the low 32 - e bits of b: 2^32 = -1
+    __device__ __forceinline__ static V mul(V b, Tw e, const ShiftArgs &)
     {
-        if constexpr (SHIFT) return f_shl<K>(b, tw_exp<K, L>(node));
-        else return m_shoup((uint32_t)b, a.z[node], a.zp[node], (uint32_t)a.m);
+        return (V)(uint32_t)((uint32_t)b << e) - (b >> (32u - e));
     }
-    __device__ static V add(V x, V y, const ShiftArgs &a)
+    __device__ __forceinline__ static V add(V x, V y) { return x + y; }
+    __device__ __forceinline__ static V sub(V x, V y, int, const ShiftArgs &) { return x - y; }
+    __device__ __forceinline__ static V sub_fwd(V x, V y, const ShiftArgs &) { return x - y; }
+    // lo - hi + m with |hi| < 2^8 <= m; past 2^32 a large multiple of m is taken away
+    __device__ __forceinline__ static uint32_t lift(V v, const ShiftArgs &a)
     {
-        if constexpr (SHIFT) return f_add<K>(x, y);
-        else { const uint64_t s = x + y; return s >= a.m ? s - a.m : s; }
+        const uint32_t lo = (uint32_t)v, t = (uint32_t)a.m - (uint32_t)(v >> 32);
+        const uint32_t r = lo + t;
+        return r < lo ? r - a.big : r;
     }
-    __device__ static V sub(V x, V y, const ShiftArgs &a)
+    __device__ __forceinline__ static V point(V F, V G, const ShiftArgs &a)
     {
-        if constexpr (SHIFT) return f_sub<K>(x, y);
-        else return x >= y ? x - y : x + a.m - y;
+        const uint64_t p = (uint64_t)lift(F, a) * lift(G, a);
+        const V v = (V)(uint32_t)p - (V)(p >> 32);                       // modulo F_5
+        return (v >> L) - (V)(uint32_t)((uint32_t)v << (32 - L));        // N^-1 = 2^-L = -2^(32 - L)
+    }
+    __device__ __forceinline__ static uint32_t out(V v, const ShiftArgs &a)
+    {
+        const uint32_t r = lift(v, a), s = r - __umulhi(r, a.onep32) * (uint32_t)a.m;
+        return min(s, s - (uint32_t)a.m);
     }
 };
+
+// ---- modulo F_4 = 2^16 + 1 = m, signed 32-bit words ----
+template <int L> struct Ops<16, L, true> {
+    using V = int32_t;
+    using Tw = uint32_t;
+    __device__ __forceinline__ static V load(uint32_t x) { return (V)x; }
+    __device__ __forceinline__ static Tw node(uint32_t i, const ShiftArgs &) { return tw_exp<16, L>(i); }
+    __device__ __forceinline__ static V mul(V b, Tw e, const ShiftArgs &)
+    {
+        return (V)(((uint32_t)b << e) & 0xffffu) - (b >> (16u - e));
+    }
+    __device__ __forceinline__ static V add(V x, V y) { return x + y; }
+    __device__ __forceinline__ static V sub(V x, V y, int, const ShiftArgs &) { return x - y; }
+    __device__ __forceinline__ static V sub_fwd(V x, V y, const ShiftArgs &) { return x - y; }
+    __device__ __forceinline__ static uint32_t canon16(V v)             // |v >> 16| < 2^8: [0, 2^16]
+    {
+        V r = (V)((uint32_t)v & 0xffffu) - (v >> 16);
+        r = r < 0 ? r + 65537 : r;
+        return (uint32_t)(r > 65536 ? r - 65537 : r);
+    }
+    __device__ __forceinline__ static V point(V F, V G, const ShiftArgs &)
+    {
+        const uint64_t p = (uint64_t)canon16(F) * canon16(G);             // <= 2^32
+        const V v = (V)((uint32_t)p & 0xffffu) - (V)(uint32_t)(p >> 16);
+        return (v >> L) - (V)(((uint32_t)v << (16 - L)) & 0xffffu);       // N^-1 = -2^(16 - L)
+    }
+    __device__ __forceinline__ static uint32_t out(V v, const ShiftArgs &) { return canon16(v); }
+};
+
+// ---- modulo m with Shoup products (SHOUP mode): forward below 25 m (a unit
+// butterfly of levels 0..2 takes y < 4m, every level adds at most 4m),
+// inverse below 128 m < 2^30 ----
+template <int K, int L> struct Ops<K, L, false> {
+    using V = uint32_t;
+    struct Tw { uint32_t z, zp; };
+    __device__ __forceinline__ static V load(uint32_t x) { return x; }
+    __device__ __forceinline__ static Tw node(uint32_t i, const ShiftArgs &a) { return Tw{a.z[i], a.zp[i]}; }
+    __device__ __forceinline__ static V mul(V b, Tw t, const ShiftArgs &a) { return b * t.z - __umulhi(b, t.zp) * (uint32_t)a.m; }
+    __device__ __forceinline__ static V add(V x, V y) { return x + y; }
+    // products are below 2m; the inputs of inverse level j below 2^(j+1) m
+    __device__ __forceinline__ static V sub(V x, V y, int j, const ShiftArgs &a) { return x - y + ((uint32_t)a.m << (j + 1)); }
+    __device__ __forceinline__ static V sub_fwd(V x, V y, const ShiftArgs &a) { return x - y + 4 * (uint32_t)a.m; }   // y < 4m
+    __device__ __forceinline__ static V point(V F, V G, const ShiftArgs &a)
+    {
+        const uint64_t p = (uint64_t)F * G;
+        const uint64_t r = p - __umul64hi(p, a.onep) * a.m;               // [0, 2m)
+        return mul((uint32_t)r, Tw{a.ninv, a.ninvp}, a);                  // [0, 2m)
+    }
+    __device__ __forceinline__ static uint32_t out(V v, const ShiftArgs &a)
+    {
+        const uint32_t m = (uint32_t)a.m, s = v - __umulhi(v, a.onep32) * m;
+        return min(s, s - m);
+    }
+};
+
+// Levels of one pass over the thread's E elements: register bits HI - 1
+// (forward first) down to 0.  tw holds the nodes level by level, the top
+// level's E >> HI first; tw_at is the place of the node of element k at
+// register bit j.
+template <int E, int HI> __device__ __forceinline__ constexpr int tw_at(int k, int j)
+{
+    return (k >> (j + 1)) + (E >> (j + 1)) - (E >> HI);
+}
+
+template <class O, int E, int HI>
+__device__ __forceinline__ void fwd(typename O::V (&v)[E], const typename O::Tw *tw, bool first, const ShiftArgs &a)
+{
+#pragma unroll
+    for (int j = HI - 1; j >= 0; --j)
+#pragma unroll
+        for (int k = 0; k < E; ++k) {
+            if (k & (1 << j)) continue;
+            const bool one = first && (k >> (j + 1)) == 0;                // node 0: twiddle 1
+            const typename O::V x = v[k];
+            const typename O::V t = one ? v[k | (1 << j)] : O::mul(v[k | (1 << j)], tw[tw_at<E, HI>(k, j)], a);
+            v[k] = O::add(x, t);
+            v[k | (1 << j)] = O::sub_fwd(x, t, a);
+        }
+}
+
+template <class O, int E, int HI>
+__device__ __forceinline__ void inv(typename O::V (&v)[E], const typename O::Tw *tw, bool first, int j0, const ShiftArgs &a)
+{
+#pragma unroll
+    for (int j = 0; j < HI; ++j)
+#pragma unroll
+        for (int k = 0; k < E; ++k) {
+            if (k & (1 << j)) continue;
+            const bool one = first && (k >> (j + 1)) == 0;
+            const typename O::V x = v[k], y = v[k | (1 << j)], d = O::sub(x, y, j0 + j, a);
+            v[k] = O::add(x, y);
+            v[k | (1 << j)] = one ? d : O::mul(d, tw[tw_at<E, HI>(k, j)], a);
+        }
+}
 
 template <int K, int L, bool SHIFT>
 __global__ void __launch_bounds__(BLK) k_conv_shift(const __grid_constant__ ShiftArgs a)
 {
-    constexpr int N = 1 << L, P = N < 32 ? N : 32, E = N / P;
-    static_assert(E == 1 || E == 2, "N <= 64");
     using O = Ops<K, L, SHIFT>;
-    const int lane = threadIdx.x & 31;
-    const uint32_t q = (uint32_t)(lane & (P - 1));
-    const unsigned FULL = 0xffffffffu;
+    using V = typename O::V;
+    using Tw = typename O::Tw;
+    constexpr int N = 1 << L, E = N < 8 ? N : 8, T = N / E, LE = L < 3 ? L : 3, L2 = L - LE;
+    constexpr int PPW = 32 / T;                            // pairs per warp
+    constexpr int PST = N + N / 8;                         // words of a pair's exchange region: x at x + x / 8
+    __shared__ V ex[L2 > 0 ? (BLK / 32) * PPW * PST : 1];
+    const int lane = threadIdx.x & 31, q = lane & (T - 1);
+    V *S = ex + (L2 > 0 ? ((threadIdx.x >> 5) * PPW + lane / T) * PST : 0);
+    // pass 1: nodes of the top levels, the same for every thread; pass 2: this thread's
+    Tw t1[E], t2[E];
+#pragma unroll
+    for (int j = LE - 1, n = 0; j >= 0; --j)
+#pragma unroll
+        for (int i = 0; i < (E >> (j + 1)); ++i, ++n) t1[n] = O::node((uint32_t)i, a);
+    if constexpr (L2 > 0) {
+#pragma unroll
+        for (int j = L2 - 1, n = 0; j >= 0; --j)
+#pragma unroll
+            for (int i = 0; i < (E >> (j + 1)); ++i, ++n) t2[n] = O::node((uint32_t)(q * (E >> (j + 1)) + i), a);
+    }
+    auto to_rows = [&](V (&v)[E]) {                        // pass 1 layout -> pass 2 layout
+        __syncwarp();
+#pragma unroll
+        for (int k = 0; k < E; ++k) S[(q + T * k) + (q + T * k) / 8] = v[k];
+        __syncwarp();
+#pragma unroll
+        for (int k = 0; k < E; ++k) v[k] = S[9 * q + k];
+    };
     const long long gwarp = ((long long)blockIdx.x * BLK + threadIdx.x) >> 5;
     const long long nwarp = ((long long)gridDim.x * BLK) >> 5;
-    constexpr int PPW = 32 / P;                         // pairs per warp
     for (long long base = gwarp * PPW; base < a.batch; base += nwarp * PPW) {
-        const long long pair = base + lane / P;
+        const long long pair = base + lane / T;
         const bool live = pair < a.batch;
-        uint64_t v[2][E];
+        const uint32_t *f = a.f + pair * N + q, *g = a.g + pair * N + q;
+        V v[E], w[E];
 #pragma unroll
         for (int k = 0; k < E; ++k) {
-            const uint32_t x = q + (uint32_t)(P * k);
-            v[0][k] = live ? a.f[pair * N + x] : 0;
-            v[1][k] = live ? a.g[pair * N + x] : 0;
+            v[k] = O::load(live ? f[T * k] : 0u);
+            w[k] = O::load(live ? g[T * k] : 0u);
         }
-        // forward node tree, levels d = 0 .. L-1 (distance D = 2^(L-1-d))
-#pragma unroll
-        for (int d = 0; d < L; ++d) {
-            const int D = 1 << (L - 1 - d);
-#pragma unroll
-            for (int s = 0; s < 2; ++s) {
-                if (D >= P) {                               // inside the lane: elements k = 0 (a), 1 (b)
-                    const uint64_t t = O::tw(v[s][1], 0u, a);   // node (q + P k) >> (L - d) = 0 at d = 0
-                    const uint64_t x0 = v[s][0];
-                    v[s][0] = O::add(x0, t, a);
-                    v[s][1] = O::sub(x0, t, a);
-                } else {
-#pragma unroll
-                    for (int k = 0; k < E; ++k) {
-                        const uint32_t x = q + (uint32_t)(P * k);
-                        const uint32_t node = x >> (L - d);
-                        const uint64_t mine = v[s][k];
-                        const uint64_t other = __shfl_xor_sync(FULL, mine, D);
-                        v[s][k] = (q & D) ? O::sub(other, O::tw(mine, node, a), a)
-                                          : O::add(mine, O::tw(other, node, a), a);
-                    }
-                }
-            }
+        fwd<O, E, LE>(v, t1, true, a);
+        fwd<O, E, LE>(w, t1, true, a);
+        if constexpr (L2 > 0) {
+            to_rows(v);
+            fwd<O, E, L2>(v, t2, false, a);
+            to_rows(w);
+            fwd<O, E, L2>(w, t2, false, a);
         }
-        // pointwise product with N^-1
 #pragma unroll
-        for (int k = 0; k < E; ++k) {
-            if constexpr (SHIFT) {
-                const uint64_t p = f_mul<K>(v[0][k], v[1][k]);
-                const uint64_t t = f_shl<K>(p, (uint32_t)(K - L));   // 2^(K - L) = -2^-L
-                v[0][k] = t == 0 ? 0 : (1ull << K) + 1 - t;
-            } else {
-                const uint32_t m = (uint32_t)a.m;
-                const uint64_t p = (v[0][k] * v[1][k]) % m;           // operands < m < 2^24
-                v[0][k] = m_shoup((uint32_t)p, a.ninv, a.ninvp, m);
-            }
+        for (int k = 0; k < E; ++k) v[k] = O::point(v[k], w[k], a);
+        if constexpr (L2 > 0) {
+            inv<O, E, L2>(v, t2, false, 0, a);
+            __syncwarp();
+#pragma unroll
+            for (int k = 0; k < E; ++k) S[9 * q + k] = v[k];
+            __syncwarp();
+#pragma unroll
+            for (int k = 0; k < E; ++k) v[k] = S[(q + T * k) + (q + T * k) / 8];
         }
-        // inverse: transposed tree, levels d = L-1 .. 0
-#pragma unroll
-        for (int d = L - 1; d >= 0; --d) {
-            const int D = 1 << (L - 1 - d);
-            if (D >= P) {
-                const uint64_t x0 = v[0][0], x1 = v[0][1];
-                v[0][0] = O::add(x0, x1, a);
-                v[0][1] = O::tw(O::sub(x0, x1, a), 0u, a);
-            } else {
-#pragma unroll
-                for (int k = 0; k < E; ++k) {
-                    const uint32_t x = q + (uint32_t)(P * k);
-                    const uint32_t node = x >> (L - d);
-                    const uint64_t mine = v[0][k];
-                    const uint64_t other = __shfl_xor_sync(FULL, mine, D);
-                    v[0][k] = (q & D) ? O::tw(O::sub(other, mine, a), node, a) : O::add(mine, other, a);
-                }
-            }
-        }
-        // output index <-x>_N, residue modulo m
+        inv<O, E, LE>(v, t1, true, L2, a);
         if (live) {
 #pragma unroll
             for (int k = 0; k < E; ++k) {
-                const uint32_t x = q + (uint32_t)(P * k);
-                uint64_t r = v[0][k];
-                if constexpr (SHIFT) {
-                    r = r - __umul64hi(r, a.onep) * a.m;             // r <= 2^K < 2^64: Shoup by 1
-                    if (r >= a.m) r -= a.m;
-                }
-                a.h[pair * N + ((N - x) & (N - 1))] = (uint32_t)r;
+                const uint32_t x = (uint32_t)(q + T * k);
+                a.h[pair * N + ((N - x) & (N - 1))] = O::out(v[k], a);
             }
         }
     }
@@ -247,6 +316,8 @@ extern "C" ntt_status conv_circular_shift(uint64_t m, uint32_t N, const uint32_t
     ShiftArgs a{};
     a.f = f; a.g = g; a.h = h; a.batch = (long long)batch; a.m = m;
     a.onep = (uint64_t)(((unsigned __int128)1 << 64) / m);
+    a.onep32 = (uint32_t)((1ull << 32) / m);
+    a.big = (uint32_t)((1ull << 31) / m * m);
     const uint64_t w = nt::pow_mod(2, nmax / N, m);
     for (uint32_t i = 0; i < N / 2; ++i) {
         uint32_t r = 0;
@@ -259,7 +330,7 @@ extern "C" ntt_status conv_circular_shift(uint64_t m, uint32_t N, const uint32_t
     int dev = 0, nsm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    const long long pairs_per_block = (long long)(BLK / 32) * (32 / (N < 32 ? N : 32));
+    const long long pairs_per_block = (long long)BLK / (N < 8 ? 1 : N / 8);
     const long long need = ((long long)batch + pairs_per_block - 1) / pairs_per_block;
     const int grid = (int)(need < (long long)nsm * 8 ? need : (long long)nsm * 8);
     cudaStream_t st = (cudaStream_t)stream;
