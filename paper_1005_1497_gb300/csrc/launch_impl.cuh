@@ -125,19 +125,20 @@ int Launch<W>::pairs_per_block(int L, int block)
 // Rows of a convolution's split path.  Untwisted: one row of 2^LR of the
 // length-2^L tree, node twiddles from the plan's table (they depend on the
 // row).  Twisted: after the twist of the column pass the rows are whole
-// length-2^LR convolutions with the uniform table, so one kernel serves
-// every L; output lazy, natural order.
+// length-2^LR convolutions with the uniform table (OUT 1 of the column/row
+// kernel), half blocks below the longest row as for whole sequences.
 template <typename W, int L>
 static cudaError_t launch_conv_rows(bool twisted, const RowArgs<W> &a, int grid, cudaStream_t st)
 {
-    constexpr int LR = LRMax<W>::v;
-    if constexpr (L > LR && L <= Launch<W>::LMAX) {
+    if constexpr (L > LRMax<W>::v && L <= Launch<W>::LMAX) {
         if (twisted) {
-            constexpr size_t smem = CRShape<W, LR, true>::smem;
-            static const cudaError_t init = ensure_smem(k_conv_cr<W, LR, 0, 1>, smem);
+            constexpr int LR = split_row_bits<W>(L, true), BLK = row_block<W>(LR);
+            constexpr size_t smem = CRShape<W, LR, true, BLK>::smem;
+            static const cudaError_t init = ensure_smem(k_conv_cr<W, LR, 0, 1, BLK>, smem);
             if (init != cudaSuccess) return init;
-            k_conv_cr<W, LR, 0, 1><<<grid, BLOCK, smem, st>>>(a);
+            k_conv_cr<W, LR, 0, 1, BLK><<<grid, BLK, smem, st>>>(a);
         } else {
+            constexpr int LR = LRMax<W>::v;
             constexpr size_t smem = CRShape<W, LR, false>::smem;
             static const cudaError_t init = ensure_smem(k_conv_rows<W, L, LR>, smem);
             if (init != cudaSuccess) return init;
@@ -164,11 +165,10 @@ static cudaError_t launch_rows_fwd(const RowArgs<W> &a, int grid, cudaStream_t s
     }
 }
 
-// Column bits of the split path: up to CMAX in one pass; above that, a top
-// pass of L - LR - LB bits and a middle pass of LB = (L - LR) / 2 bits.
-constexpr int CMAX = 5;
-template <typename W, int L> struct ColSplit {
-    static constexpr int LR = LRMax<W>::v;
+// Row and column bits of the split path (split_row_bits).  Above CMAX column
+// bits: a top pass of L - LR - LB bits and a middle pass of LB = (L - LR) / 2.
+template <typename W, int L, bool TW> struct ColSplit {
+    static constexpr int LR = split_row_bits<W>(L, TW);
     static constexpr int LC = L - LR;
     static constexpr bool TWO = LC > CMAX;
     static constexpr int LB = TWO ? LC / 2 : 0;          // middle bits
@@ -178,10 +178,11 @@ template <typename W, int L> struct ColSplit {
 template <typename W, int L, int NS, int SRC, bool TW>
 static cudaError_t launch_cols_fwd(const ColArgs<W> &a, cudaStream_t st)
 {
-    using CS = ColSplit<W, L>;
-    if constexpr (L > CS::LR && L <= Launch<W>::LMAX) {
-        const long long threads = a.npairs << CS::TOPLR;
-        k_cols_fwd<W, L, CS::TOPLR, NS, SRC, TW && !CS::TWO><<<(int)((threads + 255) / 256), 256, 0, st>>>(a);
+    using CS = ColSplit<W, L, TW>;
+    if constexpr (L > LRMax<W>::v && L <= Launch<W>::LMAX) {
+        constexpr bool TWIST = TW && !CS::TWO;
+        const long long threads = a.npairs * (cols_both<W, NS, TWIST>() ? 1 : NS) << CS::TOPLR;
+        k_cols_fwd<W, L, CS::TOPLR, NS, SRC, TWIST><<<(int)((threads + COLB - 1) / COLB), COLB, 0, st>>>(a);
         if constexpr (CS::TWO) {
             const long long t2 = a.npairs << (L - CS::LB);
             k_cols_mid_fwd<W, L, CS::LR, CS::LB, NS, TW><<<(int)((t2 + 255) / 256), 256, 0, st>>>(a);
@@ -195,17 +196,17 @@ static cudaError_t launch_cols_fwd(const ColArgs<W> &a, cudaStream_t st)
 template <typename W, int L, int DST, bool TW>
 static cudaError_t launch_cols_inv(const ColArgs<W> &a, cudaStream_t st)
 {
-    using CS = ColSplit<W, L>;
-    if constexpr (L > CS::LR && L <= Launch<W>::LMAX) {
+    using CS = ColSplit<W, L, TW>;
+    if constexpr (L > LRMax<W>::v && L <= Launch<W>::LMAX) {
         if constexpr (CS::TWO) {
             const long long t2 = a.npairs << (L - CS::LB);
             k_cols_mid_inv<W, L, CS::LR, CS::LB, TW><<<(int)((t2 + 255) / 256), 256, 0, st>>>(a);
         }
         const long long threads = a.npairs << CS::TOPLR;
-        if constexpr (sizeof(W) == 4 && L - CS::TOPLR == 5)
-            k_cols_inv5<W, L, CS::TOPLR, DST, TW && !CS::TWO><<<(int)((threads + 255) / 256), 256, 0, st>>>(a);
-        else
-            k_cols_inv<W, L, CS::TOPLR, DST, TW && !CS::TWO><<<(int)((threads + 255) / 256), 256, 0, st>>>(a);
+        const int grid = (int)((threads + COLB - 1) / COLB);
+        constexpr int ROW = TW ? CS::LR : 0;
+        if constexpr (sizeof(W) == 4 && L - CS::TOPLR == 5) k_cols_inv5<W, L, CS::TOPLR, DST, TW && !CS::TWO, ROW><<<grid, COLB, 0, st>>>(a);
+        else k_cols_inv<W, L, CS::TOPLR, DST, TW && !CS::TWO, ROW><<<grid, COLB, 0, st>>>(a);
         return launched(CS::TWO ? 2 : 1);
     } else {
         return cudaErrorInvalidValue;
@@ -321,15 +322,27 @@ cudaError_t Launch<W>::rows_fwd(int L, const RowArgs<W> &a, int grid, cudaStream
 #undef C
 }
 
-template <typename W>
-cudaError_t Launch<W>::rows_uni(const RowArgs<W> &a, int grid, cudaStream_t st)
+template <typename W, int L>
+static cudaError_t launch_rows_uni(const RowArgs<W> &a, int grid, cudaStream_t st)
 {
-    constexpr int LR = LRMax<W>::v;
-    constexpr size_t smem = TwBytes<W, LR>::v + RowShape<W, LR, LR>::smem(1);
-    static const cudaError_t init = ensure_smem(k_rows_uni<W, LR>, smem);
-    if (init != cudaSuccess) return init;
-    k_rows_uni<W, LR><<<grid, BLOCK, smem, st>>>(a);
-    return launched();
+    if constexpr (L > LRMax<W>::v && L <= Launch<W>::LMAX) {
+        constexpr int LR = split_row_bits<W>(L, true);
+        constexpr size_t smem = TwBytes<W, LR>::v + RowShape<W, LR, LR>::smem(1);
+        static const cudaError_t init = ensure_smem(k_rows_uni<W, LR>, smem);
+        if (init != cudaSuccess) return init;
+        k_rows_uni<W, LR><<<grid, BLOCK, smem, st>>>(a);
+        return launched();
+    } else {
+        return cudaErrorInvalidValue;
+    }
+}
+
+template <typename W>
+cudaError_t Launch<W>::rows_uni(int L, const RowArgs<W> &a, int grid, cudaStream_t st)
+{
+#define C(X) launch_rows_uni<W, X>(a, grid, st)
+    NTT_SWITCH_L(C)
+#undef C
 }
 
 template <typename W>

@@ -88,7 +88,8 @@ struct ntt_plan_s {
     ModC<uint32_t> c32{};
     ModC<uint64_t> c64{};
     bool split = false;
-    int LR = 0;
+    int LR = 0;                        // split path: log2 of the row length, row-twiddle form
+    int LRT = 0;                       // and twist form
     uint32_t wave = 0;                 // pairs per scratch wave (split path)
     bool twist = false;                // split path form: the four-step twist (else row-dependent twiddles)
     int block = ntt::BLOCK;            // whole sequences: threads per block of the fused kernel
@@ -96,7 +97,7 @@ struct ntt_plan_s {
     void *scratch = nullptr;           // 2 * wave * N words
     void *pd = nullptr;                // split path, one column pass: the scaled twist factor of element x, at x
     void *pw = nullptr;                // split path, two column passes: (w^e, Shoup quotient), e < N
-    void *pwl = nullptr;               // and (scaled w^(s l), quotient) at s 32 + l, s < 2^(L - LR), l < 32
+    void *pwl = nullptr;               // and (scaled w^(s l), quotient) at s 32 + l, s < 2^(L - LRT), l < 32
     uint64_t twist_unscale = 1;        // inverse of the scale that the twist's factors carry
     int nsm = 1;
     int device = 0;
@@ -176,6 +177,7 @@ extern "C" ntt_status ntt_plan(uint64_t m, uint32_t N, ntt_plan_t *out)
     const int lrmax = word == 32 ? Launch<uint32_t>::LRMAX : Launch<uint64_t>::LRMAX;
     p->split = L > lrmax;
     p->LR = p->split ? lrmax : L;
+    p->LRT = !p->split ? L : word == 32 ? ntt::split_row_bits<uint32_t>(L, true) : ntt::split_row_bits<uint64_t>(L, true);
     if (!p->split) p->block = ntt_default_block(word, L);
     if (!p->split)                                      // one block per pair below this batch (host_sched.h)
         p->small_max = ntt::small_batch_max(L, (word == 32 ? ntt::Arith<uint32_t>::RB : ntt::Arith<uint64_t>::RB) + 5,
@@ -257,13 +259,13 @@ extern "C" ntt_status ntt_plan(uint64_t m, uint32_t N, ntt_plan_t *out)
                 memcpy(&t[2 * i * elt], a, sizeof a);
             }
         };
-        if (L - p->LR <= 5) {
-            // one column pass: element x = t + k 2^LR (t < 2^LR, k < 2^(L-LR))
+        if (L - p->LRT <= ntt::CMAX) {
+            // one column pass: element x = t + k 2^LR (t < 2^LR, k < 2^(L-LR), LR = LRT)
             // takes s w^(brv(k) t), the same for every pair, so the factor is
             // stored at x and read in the data's own (coalesced) layout
-            const int lc = L - p->LR;
+            const int lc = L - p->LRT;
             for (size_t x = 0; x < N; ++x) {
-                const size_t k = x >> p->LR, t = x & (((size_t)1 << p->LR) - 1);
+                const size_t k = x >> p->LRT, t = x & (((size_t)1 << p->LRT) - 1);
                 put(tab, x, all[((nt::bit_reverse(k, lc) * t) % N * (nmax / N) + se) % nmax]);
             }
             if (!ntt::dev_alloc(&p->pd, tab.size())) return ntt_fail(NTT_ERR_OOM, "ntt_plan: twist diagonal");
@@ -273,7 +275,7 @@ extern "C" ntt_status ntt_plan(uint64_t m, uint32_t N, ntt_plan_t *out)
             for (size_t e = 0; e < N; ++e) put(tab, e, all[e * (nmax / N)]);
             if (!ntt::dev_alloc(&p->pw, tab.size())) return ntt_fail(NTT_ERR_OOM, "ntt_plan: power table");
             CUDA_TRY(cudaMemcpy(p->pw, tab.data(), tab.size(), cudaMemcpyHostToDevice), "ntt_plan: upload powers");
-            const size_t ns = (size_t)1 << (L - p->LR);
+            const size_t ns = (size_t)1 << (L - p->LRT);
             std::vector<unsigned char> lt(2 * ns * 32 * elt);
             for (size_t sidx = 0; sidx < ns; ++sidx)
                 for (size_t l = 0; l < 32; ++l) put(lt, sidx * 32 + l, all[((sidx * l) % N * (nmax / N) + se) % nmax]);
@@ -340,9 +342,11 @@ static cudaError_t conv_dispatch(ntt_plan_t p, const W *f, const W *g, W *h, con
                       (const W *)p->pwl, (const W *)p->pd};
         cudaError_t e = Launch<W>::cols_fwd(p->L, 2, mode, tw_form, ca, st);
         if (e != cudaSuccess) return e;
-        const long long rows = np << (p->L - p->LR);
+        const int lr = tw_form ? p->LRT : p->LR, block = tw_form ? ntt::row_block<W>(lr) : ntt::BLOCK;
+        const long long rows = np << (p->L - lr);
         RowArgs<W> ra{scratch, scratch + (size_t)wave * N, scratch, nullptr, rows, 0, tw, c};
-        e = Launch<W>::conv_rows_split(p->L, tw_form, ra, row_grid(p->nsm, rows, Launch<W>::pairs_per_block(p->LR)), st);
+        const int grid = row_grid(p->nsm, rows, Launch<W>::pairs_per_block(lr, block), ntt::BLOCK / block);
+        e = Launch<W>::conv_rows_split(p->L, tw_form, ra, grid, st);
         if (e != cudaSuccess) return e;
         e = Launch<W>::cols_inv(p->L, mode, tw_form, ca, st);
         if (e != cudaSuccess) return e;
@@ -371,10 +375,11 @@ static cudaError_t ntt_dispatch(ntt_plan_t p, const W *x, W *y, long long batch,
                       (const W *)p->pwl, (const W *)p->pd};
         cudaError_t e = Launch<W>::cols_fwd(p->L, 1, 0, twisted, ca, st);
         if (e != cudaSuccess) return e;
-        const long long rows = np << (p->L - p->LR);
+        const int lr = twisted ? p->LRT : p->LR;
+        const long long rows = np << (p->L - lr);
         RowArgs<W> ra{scratch, nullptr, nullptr, nullptr, rows, 0, tw, c};
-        const int grid = row_grid(p->nsm, rows, Launch<W>::rows_per_block(p->LR));
-        e = twisted ? Launch<W>::rows_uni(ra, grid, st) : Launch<W>::rows_fwd(p->L, ra, grid, st);
+        const int grid = row_grid(p->nsm, rows, Launch<W>::rows_per_block(lr));
+        e = twisted ? Launch<W>::rows_uni(p->L, ra, grid, st) : Launch<W>::rows_fwd(p->L, ra, grid, st);
         if (e != cudaSuccess) return e;
         ModC<W> cs = c;                                // the output factor: N^-1, and the twist's scale undone
         const uint64_t sc = nt::mul_mod(inv ? p->n_inv : 1, twisted ? p->twist_unscale : 1, p->m);

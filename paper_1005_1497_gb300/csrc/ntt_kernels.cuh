@@ -405,10 +405,10 @@ __device__ __forceinline__ void cols_from_rows(const W *S, uint32_t stride, uint
 // list), by blocks (ntt_block.cuh).
 // Rows [base + row group, end) by steps of stride; end is a.nrows unless ITEM.
 // OUT 0: canonical, at block_out(x) (a whole convolution); OUT 1: lazy
-// residues of a row of a convolution's split path, after the twist: element
-// 4 t' + r goes to <4 t' - r>, where the transposed column pass reads it (its
-// output stage reverses the whole index); the factor 2^(B + BB) / N is in
-// the twist's diagonal.
+// residues of a row of a convolution's split path, after the twist, stored
+// in place: position 4 t' + r holds the inverse's element <4 t' - r> of the
+// row (row_element below; the transposed column pass accounts for it); the
+// factor 2^(B + BB) / N is in the twist's diagonal.
 template <typename W, int L, int SRC, bool ITEM = false, int OUT = 0, class X = NoExact, int BLK = BLOCK>
 __device__ __forceinline__ void conv_cr_body(const RowArgs<W> &a, long long base, long long stride, long long end = 0,
                                              const ExactArgs *xa = nullptr)
@@ -577,8 +577,7 @@ __device__ __forceinline__ void conv_cr_body(const RowArgs<W> &a, long long base
 #pragma unroll
                 for (int e = 0; e < VEC; ++e) t[e] = v[0][(j * VEC + e) * RC + k];
                 if constexpr (OUT == 1) {
-#pragma unroll
-                    for (int e = 0; e < VEC; ++e) hcur[(x + e - 2 * ((x + e) & 3u)) & (N - 1u)] = t[e];
+                    st_vec<W, VEC>(hcur + x, t, true);      // scratch rows: aligned
                 } else {
 #pragma unroll
                     for (int e = 0; e < VEC; ++e) t[e] = canon<W>(t[e], a.c.cB, a.c.cBp, a.c.m);
@@ -860,6 +859,14 @@ template <typename W> struct ColArgs {
     const W *pd;        // one column pass: (w^(brv(k) t), quotient) at x = t + k 2^LR
 };
 
+// The row element that position p of a row of 2^LR holds after the rows of
+// the twist form (OUT 1 of the column/row kernel).
+template <int LR>
+__device__ __forceinline__ uint32_t row_element(uint32_t p)
+{
+    return (p - 2 * (p & ((1u << BB) - 1u))) & ((1u << LR) - 1u);
+}
+
 // The four-step twist, one of the two forms of the split path of
 // convolutions and natural-order transforms (the plan picks one per word
 // size and length; the autotuner measures both).  In the other form the rows
@@ -973,17 +980,31 @@ __device__ __forceinline__ void col_fwd_levels(W (&v)[1 << (L - LR)], const W *_
     }
 }
 
-// (the twisted 32-bit form holds f and g at once: at most 80 registers keep
-// three blocks, 24 warps, on an SM for the loads in flight)
+// Column kernels run blocks of COLB threads and are bound by memory latency:
+// what counts is how many warps have their loads in flight, so each form has
+// a register cap that sets them.  Measured on GB300 (64 x 2^19 unless said;
+// 128-thread blocks against 256: 2-3%, small batches 6%, less of a last wave
+// is empty):
+//  - f and g together (the twisted 32-bit form, so that each factor is
+//    loaded once): 96 registers, five blocks, 83.8 us, 0.94 of the copy rate
+//    (six, 80 registers and spills: 86.1; four: 84.9);
+//  - otherwise one thread per sequence and column: 64-bit words 84 -> 63 us
+//    at 128 x 2^16 against a loop over f and g.
+constexpr int COLB = 128;
+template <typename W, int NS, bool TWIST> __host__ __device__ constexpr bool cols_both() { return TWIST && NS == 2 && sizeof(W) == 4; }
+template <typename W, bool BOTH, int RC>
+__host__ __device__ constexpr int cols_fwd_regs() { return BOTH ? 96 : sizeof(W) == 4 ? 128 : RC <= 16 ? 80 : 168; }
+
 template <typename W, int L, int LR, int NS, int SRC, bool TWIST>
-__global__ void __launch_bounds__(256, (TWIST && NS == 2 && sizeof(W) == 4) ? 3 : 1)
+__global__ void __maxnreg__((cols_fwd_regs<W, cols_both<W, NS, TWIST>(), (1 << (L - LR))>()))
     k_cols_fwd(const __grid_constant__ ColArgs<W> a)
 {
     constexpr int RC = 1 << (L - LR);
     constexpr uint32_t N = 1u << L;
     const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= a.npairs << LR) return;
-    const long long pw = idx >> LR;
+    constexpr bool BOTH = cols_both<W, NS, TWIST>();
+    if (idx >= (BOTH ? a.npairs : NS * a.npairs) << LR) return;
+    const long long seq = idx >> LR, pw = BOTH || NS == 1 ? seq : seq >> 1;
     const uint32_t col = (uint32_t)idx & ((1u << LR) - 1u);
     auto source = [&](int s) -> const W * {
         if constexpr (SRC == 1) {
@@ -993,7 +1014,7 @@ __global__ void __launch_bounds__(256, (TWIST && NS == 2 && sizeof(W) == 4) ? 3 
             return (s == 0 ? a.src0 : a.src1) + (size_t)(a.pair0 + pw) * N;
         }
     };
-    if constexpr (TWIST && NS == 2 && sizeof(W) == 4) {
+    if constexpr (BOTH) {
         // 32-bit words: f and g together, so that each twist factor is
         // loaded once for both
         const W *sf = source(0), *sg = source(1);
@@ -1015,37 +1036,36 @@ __global__ void __launch_bounds__(256, (TWIST && NS == 2 && sizeof(W) == 4) ? 3 
             dg[x] = csub<W>(shoup<W>(vg[k], z, zp, a.c.m), a.c.m);
         }
     } else {
-#pragma unroll 1
-        for (int s = 0; s < NS; ++s) {
-            const W *src = source(s);
-            W *dst = (s == 0 ? a.dst0 : a.dst1) + (size_t)pw * N;
-            W v[RC];
+        const int s = NS == 1 ? 0 : (int)(seq & 1);
+        const W *src = source(s);
+        W *dst = (s == 0 ? a.dst0 : a.dst1) + (size_t)pw * N;
+        W v[RC];
 #pragma unroll
-            for (int k = 0; k < RC; ++k) v[k] = src[col + ((uint32_t)k << LR)];
-            col_fwd_levels<W, L, LR, L - LR - 1>(v, a.tw, a.c);
-            if constexpr (TWIST) {
+        for (int k = 0; k < RC; ++k) v[k] = src[col + ((uint32_t)k << LR)];
+        col_fwd_levels<W, L, LR, L - LR - 1>(v, a.tw, a.c);
+        if constexpr (TWIST) {
 #pragma unroll
-                for (int k = 0; k < RC; ++k) {
-                    W z, zp;
-                    ld_pair_g<W>(a.pd + 2 * (size_t)(col + ((uint32_t)k << LR)), z, zp);
-                    v[k] = csub<W>(shoup<W>(v[k], z, zp, a.c.m), a.c.m);
-                    // 64-bit words: keep the compiler from hoisting every table
-                    // load ahead of the products (it spills them otherwise)
-                    if constexpr (sizeof(W) == 8 && RC > 8)
-                        if ((k & 7) == 7) asm volatile("" ::: "memory");
-                }
+            for (int k = 0; k < RC; ++k) {
+                W z, zp;
+                ld_pair_g<W>(a.pd + 2 * (size_t)(col + ((uint32_t)k << LR)), z, zp);
+                v[k] = csub<W>(shoup<W>(v[k], z, zp, a.c.m), a.c.m);
+                // 64-bit words: keep the compiler from hoisting every table
+                // load ahead of the products (it spills them otherwise)
+                if constexpr (sizeof(W) == 8 && RC > 8)
+                    if ((k & 7) == 7) asm volatile("" ::: "memory");
             }
-#pragma unroll
-            for (int k = 0; k < RC; ++k) dst[col + ((uint32_t)k << LR)] = v[k];
         }
+#pragma unroll
+        for (int k = 0; k < RC; ++k) dst[col + ((uint32_t)k << LR)] = v[k];
     }
 }
 
 // Transposed top levels of the split path on column c (elements
 // x = c + k 2^LR): node twiddles k >> (J + 1), the same for every column.
 // Inputs < 2m; then the output stage: index <-x>_N, canonical residue.
-// DST 0: contiguous out; 1: descriptor h.
-template <typename W, int L, int LR, int DST, bool TWIST>
+// DST 0: contiguous out; 1: descriptor h.  ROW: log2 of the row length whose
+// positions row_element maps (the twist form's), or 0 for rows in order.
+template <typename W, int L, int LR, int DST, bool TWIST, int ROW>
 __device__ __forceinline__ void cols_inv_body(const ColArgs<W> &a)
 {
     constexpr int LC = L - LR, RC = 1 << LC;
@@ -1061,11 +1081,13 @@ __device__ __forceinline__ void cols_inv_body(const ColArgs<W> &a)
     W v[RC];
 #pragma unroll
     for (int k = 0; k < RC; ++k) v[k] = src[col + ((uint32_t)k << LR)];
+    uint32_t c = col;                                    // the column's own index
+    if constexpr (ROW > 0) c = (col & ~((1u << ROW) - 1u)) | row_element<ROW>(col & ((1u << ROW) - 1u));
     if constexpr (TWIST) {
 #pragma unroll
         for (int k = 0; k < RC; ++k) {
             W z, zp;
-            ld_pair_g<W>(a.pd + 2 * (size_t)(col + ((uint32_t)k << LR)), z, zp);
+            ld_pair_g<W>(a.pd + 2 * (size_t)(c + ((uint32_t)k << LR)), z, zp);
             v[k] = shoup<W>(v[k], z, zp, a.c.m);
             if constexpr (sizeof(W) == 8 && RC > 8)
                 if ((k & 7) == 7) asm volatile("" ::: "memory");
@@ -1074,28 +1096,23 @@ __device__ __forceinline__ void cols_inv_body(const ColArgs<W> &a)
     colg_levels<W, LC, 0, 0, 0, TW_GLOBAL, RC>(v, 0u, a.tw, a.c);
 #pragma unroll
     for (int k = 0; k < RC; ++k) {
-        const uint32_t x = col + ((uint32_t)k << LR);
+        const uint32_t x = c + ((uint32_t)k << LR);
         out[(N - x) & (N - 1u)] = csub<W>(v[k], a.c.m);
     }
 }
 
-template <typename W, int L, int LR, int DST, bool TWIST>
-__global__ void __launch_bounds__(256) k_cols_inv(const __grid_constant__ ColArgs<W> a)
+template <typename W, int L, int LR, int DST, bool TWIST, int ROW = 0>
+__global__ void __maxnreg__(sizeof(W) == 8 ? 128 : 40) k_cols_inv(const __grid_constant__ ColArgs<W> a)
 {
-    cols_inv_body<W, L, LR, DST, TWIST>(a);
+    cols_inv_body<W, L, LR, DST, TWIST, ROW>(a);
 }
 
-// The same with at most 48 registers, five blocks per SM for the loads in
-// flight: used for 32-bit words with five column bits, where the plain bound
-// takes 56 registers with contiguous output and 58 with descriptor output
-// (four blocks); measured on GB300 1.7% faster for 64 x 2^19 (contiguous)
-// and 12-14% faster for 714 x 2^19 (descriptors).  (An explicit bound raises
-// the register count of the shorter and 64-bit forms instead, so they keep
-// the plain one.)
-template <typename W, int L, int LR, int DST, bool TWIST>
-__global__ void __launch_bounds__(256, 5) k_cols_inv5(const __grid_constant__ ColArgs<W> a)
+// The same for 32-bit words with five column bits: 72 registers, seven
+// blocks per SM (512 x 2^16: 48.3 us; 48 registers, ten blocks: 52.4; 64: 49.8).
+template <typename W, int L, int LR, int DST, bool TWIST, int ROW = 0>
+__global__ void __maxnreg__(72) k_cols_inv5(const __grid_constant__ ColArgs<W> a)
 {
-    cols_inv_body<W, L, LR, DST, TWIST>(a);
+    cols_inv_body<W, L, LR, DST, TWIST, ROW>(a);
 }
 
 // Split path with more column bits than one thread holds (L - LR > 5):
@@ -1153,7 +1170,7 @@ __global__ void __launch_bounds__(256) k_cols_mid_inv(const __grid_constant__ Co
         const uint32_t hbrv = __brev(hi) >> (32 - (L - BLO - LB));
 #pragma unroll
         for (int k = 0; k < RC; ++k)
-            v[k] = twist<W, L>(v[k], (brv_c32<LB>((uint32_t)k) << (L - BLO - LB)) | hbrv, lo, a, a.pwl);
+            v[k] = twist<W, L>(v[k], (brv_c32<LB>((uint32_t)k) << (L - BLO - LB)) | hbrv, row_element<BLO>(lo), a, a.pwl);
     }
     colg_levels<W, LB, 0, 0, L - BLO - LB, TW_GLOBAL, RC>(v, hi << LB, a.tw, a.c);
 #pragma unroll

@@ -8,6 +8,29 @@
 
 namespace ntt {
 
+constexpr int CMAX = 5;                        // column bits of one pass of the split path
+
+// log2 of the split path's row length (L > LRMax).  The column passes are
+// bound by memory and the rows by arithmetic, so the twist form gives the
+// columns more levels than the longest rows would leave them: five bits for
+// 32-bit words, four for 64-bit ones (whose five-bit columns take 168
+// registers), five where four would need the longest row, whose block fills
+// an SM; never rows shorter than the column/row lengths.  Measured on GB300
+// (conv_circular, 2, 3, 4, 5 column bits at most): 32-bit 512 x 2^16 322,
+// 307, 299, 294 us and its ntt_forward 190, 188, 168, 157; 64-bit 128 x 2^16
+// 278 (2), 259, 248, 263; 12 x 2^17 80 (2), 71, 71, 60.  The row-twiddle form
+// keeps the longest rows.
+template <typename W> constexpr int split_row_bits(int L, bool twisted)
+{
+    const int lo = Arith<W>::RB + 6, hi = LRMax<W>::v;     // the column/row lengths
+    int lr = L - (sizeof(W) == 4 ? CMAX : CMAX - 1);
+    if (lr >= hi) lr = L - CMAX;
+    return !twisted || lr > hi ? hi : lr < lo ? lo : lr;
+}
+
+// Threads per block of the twist form's row kernel.
+template <typename W> constexpr int row_block(int LR) { return LR < LRMax<W>::v ? BLOCK_HALF : BLOCK; }
+
 template <typename W> struct Launch {
     static constexpr int LRMAX = LRMax<W>::v;
     static constexpr int LMAX = 20;            // split path: LMAX - LRMAX column bits, in two passes above 5
@@ -34,8 +57,8 @@ template <typename W> struct Launch {
     static cudaError_t cols_fwd(int L, int ns, int src, bool twisted, const ColArgs<W> &a, cudaStream_t st);
     static cudaError_t cols_inv(int L, int dst, bool twisted, const ColArgs<W> &a, cudaStream_t st);
     static cudaError_t rows_fwd(int L, const RowArgs<W> &a, int grid, cudaStream_t st);
-    // rows of the twist form for transforms: whole length-2^LRMAX trees in place
-    static cudaError_t rows_uni(const RowArgs<W> &a, int grid, cudaStream_t st);
+    // rows of the twist form for transforms: whole trees of the row length in place
+    static cudaError_t rows_uni(int L, const RowArgs<W> &a, int grid, cudaStream_t st);
     static cudaError_t bitrev_out(int L, bool inv, const W *src, W *dst, long long batch, const ModC<W> &c,
                                   cudaStream_t st);
     // natural-order transform of whole sequences (L <= LRMAX)
