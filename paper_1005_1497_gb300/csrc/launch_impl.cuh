@@ -217,10 +217,41 @@ template <typename W, int L, bool INV>
 static cudaError_t launch_ntt_full(const NttArgs<W> &a, int grid, cudaStream_t st)
 {
     if constexpr (L <= LRMax<W>::v) {
-        constexpr size_t smem = TwBytes<W, L>::v + RowShape<W, L, L>::smem(1);
+        constexpr size_t smem = NttShape<W, L>::smem;
         static const cudaError_t init = ensure_smem(k_ntt_rows<W, L, INV>, smem);
         if (init != cudaSuccess) return init;
         k_ntt_rows<W, L, INV><<<grid, BLOCK, smem, st>>>(a);
+        return launched();
+    } else {
+        return cudaErrorInvalidValue;
+    }
+}
+
+// Whether the twist form's transforms of length 2^L write their natural order
+// from the rows: tiles of at least four rows (with two, 64-bit 2^16, it
+// measured slower than the bit-reversal pass: 110 against 118 us at 128).
+template <typename W> constexpr bool rows_out_len(int L)
+{
+    if (L <= LRMax<W>::v || L > Launch<W>::LMAX || L - split_row_bits<W>(L, true) > CMAX) return false;
+    const int gpc = BLOCK >> (split_row_bits<W>(L, true) - Arith<W>::RB);
+    return gpc >= 4;
+}
+
+template <typename W>
+int Launch<W>::rows_out_rows(int L)
+{
+    return rows_out_len<W>(L) ? rows_per_block(split_row_bits<W>(L, true)) : 0;
+}
+
+template <typename W, int L, bool INV>
+static cudaError_t launch_rows_out(const NttArgs<W> &a, int grid, cudaStream_t st)
+{
+    if constexpr (rows_out_len<W>(L)) {
+        constexpr int LR = split_row_bits<W>(L, true);
+        constexpr size_t smem = RowsOutShape<W, L, LR>::smem;
+        static const cudaError_t init = ensure_smem(k_rows_out<W, L, LR, INV>, smem);
+        if (init != cudaSuccess) return init;
+        k_rows_out<W, L, LR, INV><<<grid, BLOCK, smem, st>>>(a);
         return launched();
     } else {
         return cudaErrorInvalidValue;
@@ -327,7 +358,7 @@ static cudaError_t launch_rows_uni(const RowArgs<W> &a, int grid, cudaStream_t s
 {
     if constexpr (L > LRMax<W>::v && L <= Launch<W>::LMAX) {
         constexpr int LR = split_row_bits<W>(L, true);
-        constexpr size_t smem = TwBytes<W, LR>::v + RowShape<W, LR, LR>::smem(1);
+        constexpr size_t smem = NttShape<W, LR>::smem;
         static const cudaError_t init = ensure_smem(k_rows_uni<W, LR>, smem);
         if (init != cudaSuccess) return init;
         k_rows_uni<W, LR><<<grid, BLOCK, smem, st>>>(a);
@@ -406,6 +437,19 @@ cudaError_t Launch<W>::ntt_full(int L, bool inv, const NttArgs<W> &a, int grid, 
 #undef C
     }
 #define C(X) launch_ntt_full<W, X, false>(a, grid, st)
+    NTT_SWITCH_L(C)
+#undef C
+}
+
+template <typename W>
+cudaError_t Launch<W>::rows_out(int L, bool inv, const NttArgs<W> &a, int grid, cudaStream_t st)
+{
+    if (inv) {
+#define C(X) launch_rows_out<W, X, true>(a, grid, st)
+        NTT_SWITCH_L(C)
+#undef C
+    }
+#define C(X) launch_rows_out<W, X, false>(a, grid, st)
     NTT_SWITCH_L(C)
 #undef C
 }

@@ -8,4 +8,6 @@ template cudaError_t Launch<uint64_t>::plain(int, const uint64_t *, const uint64
                                              long long, const uint64_t *, const ModC<uint64_t> &, int, cudaStream_t);
 template cudaError_t Launch<uint64_t>::check_range(const uint64_t *, long long, uint64_t, unsigned long long *, int,
                                                    cudaStream_t);
+template int Launch<uint64_t>::rows_out_rows(int);
+template cudaError_t Launch<uint64_t>::rows_out(int, bool, const NttArgs<uint64_t> &, int, cudaStream_t);
 }  // namespace ntt

@@ -377,14 +377,26 @@ static cudaError_t ntt_dispatch(ntt_plan_t p, const W *x, W *y, long long batch,
         if (e != cudaSuccess) return e;
         const int lr = twisted ? p->LRT : p->LR;
         const long long rows = np << (p->L - lr);
-        RowArgs<W> ra{scratch, nullptr, nullptr, nullptr, rows, 0, tw, c};
-        const int grid = row_grid(p->nsm, rows, Launch<W>::rows_per_block(lr));
-        e = twisted ? Launch<W>::rows_uni(p->L, ra, grid, st) : Launch<W>::rows_fwd(p->L, ra, grid, st);
-        if (e != cudaSuccess) return e;
         ModC<W> cs = c;                                // the output factor: N^-1, and the twist's scale undone
         const uint64_t sc = nt::mul_mod(inv ? p->n_inv : 1, twisted ? p->twist_unscale : 1, p->m);
         cs.ninv = (W)sc;
         cs.ninvp = (W)nt::shoup_quot(sc, p->m, (int)sizeof(W) * 8);
+        // From 32 tiles on the rows write the natural order themselves:
+        // measured faster on GB300 at every size from there (16 x 2^15 11.9 ->
+        // 10.8 us, 512 x 2^16 156 -> 134 us, 64-bit 512 x 2^14 94 -> 88 us).
+        // Below, a handful of SMs would write everything; the bit-reversal
+        // pass spreads the output over all of them.
+        const int per = twisted ? Launch<W>::rows_out_rows(p->L) : 0;
+        if (per && rows / per >= 32) {
+            NttArgs<W> na{scratch, y + (size_t)w0 * N, np, tw, cs};
+            e = Launch<W>::rows_out(p->L, inv, na, (int)std::min<long long>(rows / per, p->nsm), st);
+            if (e != cudaSuccess) return e;
+            continue;
+        }
+        RowArgs<W> ra{scratch, nullptr, nullptr, nullptr, rows, 0, tw, c};
+        const int grid = row_grid(p->nsm, rows, Launch<W>::rows_per_block(lr));
+        e = twisted ? Launch<W>::rows_uni(p->L, ra, grid, st) : Launch<W>::rows_fwd(p->L, ra, grid, st);
+        if (e != cudaSuccess) return e;
         e = Launch<W>::bitrev_out(p->L, inv, scratch, y + (size_t)w0 * N, np, cs, st);
         if (e != cudaSuccess) return e;
     }

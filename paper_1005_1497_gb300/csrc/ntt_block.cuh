@@ -67,7 +67,8 @@ __device__ __forceinline__ uint64_t mont(unsigned __int128 T, const ModC<uint64_
 // are 16-byte accesses (conflict-free: eight lanes of the contiguous layout
 // start 36 words apart) and the strided layouts stay conflict-free; all
 // others one pad word, as in Geo.  Rows of fewer than 32 threads share a
-// warp: their regions lie GS words apart, GS = T modulo the banks.
+// warp: their regions lie GS words apart, an odd multiple of T, which spreads
+// a warp's groups over all banks.
 template <typename W, int LR>
 struct BGeo : Geo<W, LR> {
     using G = Geo<W, LR>;
@@ -75,7 +76,7 @@ struct BGeo : Geo<W, LR> {
     static constexpr int PADW = VX ? 4 : 1;
     static constexpr int ROWP = G::ROW + PADW * (G::ROW >> G::PADSH);
     static constexpr int BANKS = (int)(128 / sizeof(W));
-    static constexpr int GS = G::T < BANKS ? 2 * ROWP + ((G::T - 2 * ROWP) % BANKS + BANKS) % BANKS : 2 * ROWP;
+    static constexpr int GS = G::T < BANKS ? (2 * ROWP / G::T | 1) * G::T : 2 * ROWP;
     __host__ __device__ static constexpr uint32_t pad(uint32_t x) { return x + PADW * (x >> G::PADSH); }
 };
 

@@ -94,6 +94,10 @@ __device__ __forceinline__ uint32_t shoup<uint32_t>(uint32_t b, uint32_t z, uint
     return r;
 }
 
+// The same with the factor 1: v mod m in [0, 2m), given floor(2^B / m).
+template <typename W>
+__device__ __forceinline__ W shoup_one(W v, W onep, W m) { return v - Arith<W>::mulhi(v, onep) * m; }
+
 // v in [0, 2m) -> [0, m)
 template <typename W>
 __device__ __forceinline__ W csub(W v, W m) { W t = v - m; return t < v ? t : v; }
@@ -551,6 +555,43 @@ __device__ __forceinline__ void dit_all(W (&v)[Geo<W, LR>::R], uint32_t rowoff, 
     if constexpr (P > 0) {
         exchange1<W, LR, P, P - 1>(v, S, tau, gid);
         dit_all<W, LR, P - 1, TWS>(v, rowoff, tau, S, gid, tw, c);
+    }
+}
+
+// Storing the registers of the last forward pass (layout lo = 0, element
+// bl + k, bl a multiple of R) at their bit-reversed places of a padded row,
+// and reading the natural order back in the first pass's layout, from t or
+// from <-t>_N.  Each address is one base per thread and a constant per
+// register: brv(bl + k) = brv(bl) + (brv_R(k) << (L - RL)), and -t steps
+// back by whole multiples of the first pass's stride.
+template <typename W, int L>
+__device__ __forceinline__ void scatter_reversed(const W (&v)[Geo<W, L>::R], W *S, uint32_t tau)
+{
+    using G = Geo<W, L>;
+    const uint32_t bl = G::base(G::NPASS - 1, tau);
+    const uint32_t at = G::pad(L == 0 ? 0u : __brev(bl) >> (32 - (L ? L : 1)));
+#pragma unroll
+    for (int k = 0; k < G::R; ++k) S[at + G::pad((uint32_t)brv_c<G::RL>(k) << G::TL)] = v[k];
+}
+
+template <typename W, int L, bool NEG>
+__device__ __forceinline__ void gather_natural(W (&v)[Geo<W, L>::R], const W *S, uint32_t tau)
+{
+    using G = Geo<W, L>;
+    constexpr uint32_t N = 1u << L;
+    static_assert(G::TL == 0 || G::lo(0) == G::TL, "first pass: stride T");
+    const uint32_t b0 = G::base(0, tau);
+    if constexpr (!NEG || G::TL < G::PADSH) {
+#pragma unroll
+        for (int k = 0; k < G::R; ++k) {
+            const uint32_t t = b0 + ((uint32_t)k << G::lo(0));
+            v[k] = S[G::pad(NEG ? ((N - t) & (N - 1u)) : t)];
+        }
+    } else {
+        const W *p = S + G::pad(N - b0);                      // <-t> = N - b0 - k T (b0 = k = 0: 0)
+        v[0] = S[G::pad((N - b0) & (N - 1u))];
+#pragma unroll
+        for (int k = 1; k < G::R; ++k) v[k] = p[-(int)G::pad((uint32_t)k << G::lo(0))];
     }
 }
 

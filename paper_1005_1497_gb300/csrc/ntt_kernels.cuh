@@ -59,15 +59,21 @@ struct RowShape {
 
 // Shared memory of the one-warp fused kernel: the twiddles (the first N / 8
 // pairs for lengths that convolve by blocks) and, for lengths of more than
-// one register pass, two rows per group.
+// one register pass, two rows per group and a plain one for the next f (the
+// next g goes into g's row once the products are done with it).  Measured on
+// GB300 against loading at the start of each pair: 20011 x 2^8 35.1 -> 32.2 us.
 template <typename W, int L, int BLK = BLOCK>
 struct FusedShape {
     static constexpr bool BLOCKS = L >= BLOCK_LMIN;
     using G = BGeo<W, L>;
     static constexpr int GPC = BLK / G::T;
     static constexpr int TWL = BLOCKS ? L - BB : L;     // TwBytes: 2^(TWL - 1) pairs
-    static constexpr int GS = G::NPASS > 1 ? G::GS : 0;
-    static constexpr size_t smem = TwBytes<W, TWL>::v + (size_t)GPC * GS * sizeof(W);
+    static constexpr bool STAGE = G::NPASS > 1;         // the next pair staged by asynchronous copies
+    static constexpr int GS = STAGE ? G::GS : 0;
+    // words per asynchronous copy that keep every group's rows aligned
+    static constexpr uint32_t CH = 16 / sizeof(W) > 2 && G::GS % 4 == 0 && G::ROWP % 4 == 0 ? 4 : G::GS % 2 == 0 && G::ROWP % 2 == 0 ? 2 : 1;
+    static constexpr size_t next = TwBytes<W, TWL>::v + ((size_t)GPC * GS * sizeof(W) + 15) / 16 * 16;
+    static constexpr size_t smem = next + (STAGE ? (size_t)GPC * G::ROW * sizeof(W) : 0);
 };
 
 // Hint: fetch `bytes` bytes at p into L2 with one bulk copy-engine
@@ -88,6 +94,21 @@ __device__ __forceinline__ void cp_async(void *dst, const void *src)
     else asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(d), "l"(src), "n"(BYTES) : "memory");
 }
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+// N = 2^L consecutive words by the T threads of a group, CH words per copy
+// where the source allows.
+template <typename W, int L, uint32_t CH>
+__device__ __forceinline__ void stage_seq(const W *src, W *dst, uint32_t tau)
+{
+    using G = Geo<W, L>;
+    if (CH > 1 && G::R % CH == 0 && ((uintptr_t)src & (CH * sizeof(W) - 1)) == 0) {
+#pragma unroll
+        for (uint32_t i = 0; i < G::R / CH; ++i) cp_async<CH * sizeof(W)>(dst + (tau + G::T * i) * CH, src + (tau + G::T * i) * CH);
+    } else {
+#pragma unroll 8
+        for (uint32_t i = 0; i < G::R; ++i) cp_async<sizeof(W)>(dst + tau + G::T * i, src + tau + G::T * i);
+    }
+}
 
 // Input and output of the fused bodies: plain words (the default), or the
 // ends of the exact convolution fused in -- signed 64-bit inputs reduced
@@ -138,8 +159,9 @@ __device__ __forceinline__ void st_out(W *hp, long long pair, uint32_t N, uint32
 // regions 0 and 1, multiplied block by block (ntt_block.cuh; lengths below 8
 // pointwise), and sent back through region 0 by the decimation-in-time
 // inverse; results are stored canonical.
-// At the start of each pair one thread asks the copy engine to bring the
-// next pair's f and g into L2, so their loads do not wait on HBM.
+// Each group brings its next pair by asynchronous copies while it convolves
+// this one (lengths of one register pass and the exact inputs: loads, with the
+// next pair asked into L2).
 // Rows [base + group, a.nrows) by steps of stride.
 template <typename W, int L, int SRC, class X = NoExact, int BLK = BLOCK>
 __device__ __forceinline__ void conv_fused_body(const RowArgs<W> &a, long long base, long long stride,
@@ -171,27 +193,59 @@ __device__ __forceinline__ void conv_fused_body(const RowArgs<W> &a, long long b
         }
     };
     constexpr uint32_t INB = X::IN64 ? 8u : (uint32_t)sizeof(W);     // bytes per input element
+    constexpr bool STAGE = SH::STAGE && !X::IN64;
+    W *B = reinterpret_cast<W *>(smem_raw + SH::next) + (size_t)gid * N;
+    using BG = BGeo<W, L>;
+    const W *fp, *gp, *fn = nullptr, *gn = nullptr;
+    W *hp, *hn = nullptr;
+    if constexpr (STAGE) {
+        if (base + gid < a.nrows) {
+            ptrs(base + gid, fn, gn, hn);
+            stage_seq<W, L, SH::CH>(fn, B, tau);
+            stage_seq<W, L, SH::CH>(gn, S + BG::ROWP, tau);
+            cp_async_wait();
+            group_sync<T>(gid);
+        }
+    }
     for (long long rho = base + gid; rho < a.nrows; rho += stride) {
-        const W *fp, *gp;
-        W *hp;
-        ptrs(rho, fp, gp, hp);
-        if (tau == 0 && rho + stride < a.nrows) {
-            const W *fn, *gn;
-            W *hn;
+        const bool more = rho + stride < a.nrows;
+        if constexpr (STAGE) hp = hn;
+        else ptrs(rho, fp, gp, hp);
+        if (more) {
             ptrs(rho + stride, fn, gn, hn);
-            prefetch_l2(fn, N * INB);
-            prefetch_l2(gn, N * INB);
+            if (!STAGE && tau == 0) {
+                prefetch_l2(fn, N * INB);
+                prefetch_l2(gn, N * INB);
+            }
         }
         W v[2][R];
 #pragma unroll
         for (int k = 0; k < R; ++k) {
-            v[0][k] = ld_elem<X>(fp, b0 + ((uint32_t)k << lo0), xa);
-            v[1][k] = ld_elem<X>(gp, b0 + ((uint32_t)k << lo0), xa);
+            const uint32_t x = b0 + ((uint32_t)k << lo0);
+            if constexpr (STAGE) {
+                v[0][k] = B[x];
+                v[1][k] = S[BG::ROWP + x];
+            } else {
+                v[0][k] = ld_elem<X>(fp, x, xa);
+                v[1][k] = ld_elem<X>(gp, x, xa);
+            }
+        }
+        if constexpr (STAGE) {
+            group_sync<T>(gid);
+            if (more) stage_seq<W, L, SH::CH>(fn, B, tau);
         }
         if constexpr (SH::BLOCKS) {
             bfwd_all<W, L, L, 0, true>(v, 0u, tau, S, gid, stw, a.c);
             block_products<W, R>(v, G::base(last, tau), stw, a.c);
+            if constexpr (STAGE) {
+                group_sync<T>(gid);
+                if (more) stage_seq<W, L, SH::CH>(gn, S + BG::ROWP, tau);
+            }
             bdit_all<W, L, last>(v[0], tau, S, gid, stw, a.c);
+            if constexpr (STAGE) {
+                cp_async_wait();
+                group_sync<T>(gid);
+            }
 #pragma unroll
             for (int k = 0; k < R; ++k) {
                 const uint32_t x = b0 + ((uint32_t)k << lo0);
@@ -778,64 +832,78 @@ template <typename W> struct NttArgs {
     ModC<W> c;
 };
 
+// Rows of the natural-order kernels: one row per group of T threads for the
+// exchanges, and a plain one that holds the group's next sequence, brought
+// by asynchronous copies while this one is transformed.  Measured on GB300
+// against loading it into registers: 4096 x 2^14 forward 177 -> 169 us, 2^13
+// 155 -> 147; 64-bit words 2048 x 2^13, which had no registers to spare for
+// it, 160 -> 150.  (Two groups of 512 threads with 64 registers each instead
+// of one: 226 us at 2^14; two alternating exchange rows, which need half the
+// barriers: 190 -- the warps drift apart across the unrolled code.)
+template <typename W, int L> struct NttShape {
+    using G = Geo<W, L>;
+    static constexpr int GPC = BLOCK / G::T;
+    static constexpr size_t rows = TwBytes<W, L>::v, next = rows + (size_t)GPC * G::ROWP * sizeof(W);
+    static constexpr size_t smem = next + (size_t)GPC * G::ROW * sizeof(W);
+};
+
+// One transform of the loop both kernels share: the staged sequence through
+// the forward tree, the next one's copies issued once every thread of the
+// group has read this one; v in the last pass's layout.
+template <typename W, int L, class Next>
+__device__ __forceinline__ void staged_forward(W (&v)[1][Geo<W, L>::R], const W *B, W *S, uint32_t tau, int gid, const W *stw,
+                                               const ModC<W> &c, Next next)
+{
+    using G = Geo<W, L>;
+    const uint32_t b0 = G::base(0, tau);
+#pragma unroll
+    for (int k = 0; k < G::R; ++k) v[0][k] = B[b0 + ((uint32_t)k << G::lo(0))];
+    fwd_pass<W, L, L, 0, 1, TW_SMEM, true>(v, b0, stw, c);
+    if constexpr (G::NPASS > 1) {
+        exchange<W, L, 0, 1, 1>(v, S, tau, gid);
+        next();
+        fwd_all<W, L, L, 1, 1, TW_SMEM, true>(v, 0u, tau, S, gid, stw, c);
+    } else {
+        next();                                             // (one thread per sequence)
+    }
+}
+
 template <typename W, int L, bool INV>
 __global__ void __launch_bounds__(BLOCK, 1) k_ntt_rows(const __grid_constant__ NttArgs<W> a)
 {
     using G = Geo<W, L>;
-    constexpr int T = G::T, R = G::R, GPC = RowShape<W, L, L>::GPC;
-    constexpr uint32_t N = 1u << L;
-    constexpr int last = G::NPASS - 1;
+    using SH = NttShape<W, L>;
+    constexpr int T = G::T, R = G::R, GPC = SH::GPC;
+    constexpr uint32_t N = 1u << L, Q = (uint32_t)(16 / sizeof(W));
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int gid = threadIdx.x / T;
     const uint32_t tau = threadIdx.x % T;
     W *stw = reinterpret_cast<W *>(smem_raw);
-    W *S = reinterpret_cast<W *>(smem_raw + TwBytes<W, L>::v) + (size_t)gid * G::ROWP;
-    const uint32_t b0 = G::base(0, tau), bl = G::base(last, tau);
-    constexpr int lo0 = G::lo(0), lol = G::lo(last);
+    W *S = reinterpret_cast<W *>(smem_raw + SH::rows) + (size_t)gid * G::ROWP;
+    W *B = reinterpret_cast<W *>(smem_raw + SH::next) + (size_t)gid * N;
+    const uint32_t b0 = G::base(0, tau);
     stage_twiddles<W>(a.tw, stw, TwBytes<W, L>::pairs);
-    __syncthreads();
-    const W scale = INV ? a.c.ninv : (W)1;
-    const W scalep = INV ? a.c.ninvp : a.c.onep;
-
-    // 32-bit words: the next sequence is loaded into w while this one is
-    // transformed (every group of a block otherwise waits on its loads at
-    // the same time); 64-bit words have no registers to spare for it
-    constexpr bool PF = sizeof(W) == 4;
     const long long step = (long long)gridDim.x * GPC;
     long long rho = (long long)blockIdx.x * GPC + gid;
-    W v[1][R], w[R];
-    auto load = [&](long long r, W (&dst)[R]) {
-        const W *xp = a.x + (size_t)r * N;
-#pragma unroll
-        for (int k = 0; k < R; ++k) dst[k] = xp[b0 + ((uint32_t)k << lo0)];
-    };
-    if (PF && rho < a.batch) load(rho, v[0]);
+    auto stage = [&](long long r) { if (r < a.batch) stage_seq<W, L, Q>(a.x + (size_t)r * N, B, tau); };
+    stage(rho);
+    cp_async_wait();
+    __syncthreads();
+    W v[1][R];
     for (; rho < a.batch; rho += step) {
+        staged_forward<W, L>(v, B, S, tau, gid, stw, a.c, [&] { stage(rho + step); });
+        cp_async_wait();                                    // visible after the next two barriers
+        group_sync<T>(gid);
+        scatter_reversed<W, L>(v[0], S, tau);
+        group_sync<T>(gid);
+        // output index t = b0 + k T (a warp's stores are one aligned run);
+        // the inverse takes its value from <-t>_N
+        gather_natural<W, L, INV>(v[0], S, tau);
         W *yp = a.y + (size_t)rho * N;
-        if (!PF) load(rho, v[0]);
-        const bool more = PF && rho + step < a.batch;
-        if (more) load(rho + step, w);
-        fwd_all<W, L, L, 0, 1, TW_SMEM>(v, 0u, tau, S, gid, stw, a.c);
-        group_sync<T>(gid);
 #pragma unroll
-        for (int k = 0; k < R; ++k) {
-            const uint32_t x = bl + ((uint32_t)k << lol);
-            const uint32_t u = L == 0 ? 0u : (__brev(x) >> (32 - L));
-            S[G::pad(u)] = v[0][k];
-        }
-        group_sync<T>(gid);
-#pragma unroll
-        for (int k = 0; k < R; ++k) {
-            // output index t (a warp's stores are one aligned run); the
-            // inverse takes its value from <-t>_N
-            const uint32_t t = b0 + ((uint32_t)k << lo0);
-            const uint32_t u = INV ? ((N - t) & (N - 1u)) : t;
-            yp[t] = csub<W>(shoup<W>(S[G::pad(u)], scale, scalep, a.c.m), a.c.m);
-        }
-        if (more) {
-#pragma unroll
-            for (int k = 0; k < R; ++k) v[0][k] = w[k];
-        }
+        for (int k = 0; k < R; ++k)
+            yp[b0 + ((uint32_t)k << G::lo(0))] = csub<W>(INV ? shoup<W>(v[0][k], a.c.ninv, a.c.ninvp, a.c.m)
+                                                             : shoup_one<W>(v[0][k], a.c.onep, a.c.m), a.c.m);
     }
 }
 
@@ -1210,46 +1278,103 @@ __global__ void __launch_bounds__(BLOCK, 1) k_rows_fwd(const __grid_constant__ R
 // whole length-2^LR tree with the uniform table (the first 2^(LR-1) entries
 // of the plan's table), staged in shared memory.  In place, tree order: the
 // same layout as the row-dependent rows (X(brv(k) + 2^LC brv(j)) at row k,
-// position j), so the same bit-reversal gather follows.  32-bit words load
-// the next row while this one is transformed.
+// position j), so the same bit-reversal gather follows.
 template <typename W, int LR>
 __global__ void __launch_bounds__(BLOCK, 1) k_rows_uni(const __grid_constant__ RowArgs<W> a)
 {
     using G = Geo<W, LR>;
-    constexpr int T = G::T, R = G::R, GPC = RowShape<W, LR, LR>::GPC;
+    using SH = NttShape<W, LR>;
+    constexpr int T = G::T, R = G::R, GPC = SH::GPC;
     constexpr int last = G::NPASS - 1;
+    constexpr uint32_t Q = (uint32_t)(16 / sizeof(W));
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int gid = threadIdx.x / T;
     const uint32_t tau = threadIdx.x % T;
     W *stw = reinterpret_cast<W *>(smem_raw);
-    W *S = reinterpret_cast<W *>(smem_raw + TwBytes<W, LR>::v) + (size_t)gid * G::ROWP;
+    W *S = reinterpret_cast<W *>(smem_raw + SH::rows) + (size_t)gid * G::ROWP;
+    W *B = reinterpret_cast<W *>(smem_raw + SH::next) + ((size_t)gid << LR);
     const uint32_t b0 = G::base(0, tau);
     stage_twiddles<W>(a.tw, stw, TwBytes<W, LR>::pairs);
-    __syncthreads();
-    constexpr bool PF = sizeof(W) == 4;
     const long long step = (long long)gridDim.x * GPC;
     long long rho = (long long)blockIdx.x * GPC + gid;
-    W v[1][R], w[R];
-    auto load = [&](long long r, W (&dst)[R]) {
-        const W *p = a.f + ((size_t)r << LR);
-#pragma unroll
-        for (int k = 0; k < R; ++k) dst[k] = p[b0 + ((uint32_t)k << G::lo(0))];
-    };
-    if (PF && rho < a.nrows) load(rho, v[0]);
+    auto stage = [&](long long r) { if (r < a.nrows) stage_seq<W, LR, Q>(a.f + ((size_t)r << LR), B, tau); };
+    stage(rho);
+    cp_async_wait();
+    __syncthreads();
+    W v[1][R];
     for (; rho < a.nrows; rho += step) {
-        if (!PF) load(rho, v[0]);
-        const bool more = PF && rho + step < a.nrows;
-        if (more) load(rho + step, w);
-        fwd_all<W, LR, LR, 0, 1, TW_SMEM>(v, 0u, tau, S, gid, stw, a.c);
+        staged_forward<W, LR>(v, B, S, tau, gid, stw, a.c, [&] { stage(rho + step); });
+        cp_async_wait();                                    // visible after the exchange's barriers
         // back to the first pass's layout, where a warp's stores are contiguous
-        if constexpr (last > 0) exchange<W, LR, last, 0, 1>(v, S, tau, gid);
+        exchange<W, LR, last, 0, 1>(v, S, tau, gid);
         W *p = const_cast<W *>(a.f) + ((size_t)rho << LR);
 #pragma unroll
         for (int k = 0; k < R; ++k) p[b0 + ((uint32_t)k << G::lo(0))] = v[0][k];
-        if (more) {
+    }
+}
+
+// The same rows with the natural order written straight from them: a tile is
+// the GPC rows k whose reversals brv(k) are consecutive (of one sequence),
+// one per group; after their trees a row holds X(brv(k) + 2^LC u2) for all
+// u2, so the tile is GPC consecutive words of every output run of 2^LC.
+// INV counts the tile's rows by the output residue instead (t = <-u>_N), so
+// that its runs are aligned too.  The factor a.c.ninv is the caller's (see
+// k_bitrev_out).  It saves the bit-reversal pass, a read and a write of every
+// word; GPC words of 4 bytes are a 32-byte sector for rows of 2^11 and half
+// of one for 2^12, which L2 merges.
+template <typename W, int L, int LR> struct RowsOutShape {
+    using G = Geo<W, LR>;
+    static constexpr int GPC = BLOCK / G::T, LC = L - LR;
+    // rows lie RS words apart: GPC rows x consecutive words spread over all banks
+    static constexpr int RS = G::ROWP + (int)(128 / sizeof(W)) / GPC;
+    static constexpr size_t rows = TwBytes<W, LR>::v, next = rows + ((size_t)GPC * RS * sizeof(W) + 15) / 16 * 16;
+    static constexpr size_t smem = next + (size_t)GPC * G::ROW * sizeof(W);
+};
+
+template <typename W, int L, int LR, bool INV>
+__global__ void __launch_bounds__(BLOCK, 1) k_rows_out(const __grid_constant__ NttArgs<W> a)
+{
+    using G = Geo<W, LR>;
+    using SH = RowsOutShape<W, L, LR>;
+    constexpr int T = G::T, R = G::R, GPC = SH::GPC, LC = SH::LC;
+    static_assert(GPC <= (1 << LC) && 32 % GPC == 0, "a tile lies in one sequence");
+    constexpr uint32_t Q = (uint32_t)(16 / sizeof(W)), CM = (1u << LC) - 1u, RM = (1u << LR) - 1u;
+    constexpr int TPS = (1 << LC) / GPC;                    // tiles per sequence
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int gid = threadIdx.x / T;
+    const uint32_t tau = threadIdx.x % T;
+    W *stw = reinterpret_cast<W *>(smem_raw);
+    W *rows = reinterpret_cast<W *>(smem_raw + SH::rows), *S = rows + (size_t)gid * SH::RS;
+    W *B = reinterpret_cast<W *>(smem_raw + SH::next) + ((size_t)gid << LR);
+    stage_twiddles<W>(a.tw, stw, TwBytes<W, LR>::pairs);
+    const long long tiles = a.batch * TPS;
+    auto stage = [&](long long tile) {
+        if (tile >= tiles) return;
+        const uint32_t res = (uint32_t)(tile % TPS) * GPC + gid, kap = INV ? (0u - res) & CM : res;
+        stage_seq<W, LR, Q>(a.x + ((size_t)(tile / TPS) << L) + ((size_t)(__brev(kap) >> (32 - LC)) << LR), B, tau);
+    };
+    stage(blockIdx.x);
+    cp_async_wait();
+    __syncthreads();
+    const uint32_t g = threadIdx.x % GPC, u0 = threadIdx.x / GPC;      // this thread's outputs: row g, u0 + i BLOCK / GPC
+    W v[1][R];
+    for (long long tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+        staged_forward<W, LR>(v, B, S, tau, gid, stw, a.c, [&] { stage(tile + gridDim.x); });
+        cp_async_wait();                                    // visible after the barriers below
+        group_sync<T>(gid);
+        scatter_reversed<W, LR>(v[0], S, tau);
+        __syncthreads();
+        const uint32_t res = (uint32_t)(tile % TPS) * GPC + g;
 #pragma unroll
-            for (int k = 0; k < R; ++k) v[0][k] = w[k];
+        for (int i = 0; i < R; ++i) {
+            const uint32_t o = u0 + (uint32_t)i * (BLOCK / GPC);       // output run; INV: <-u>, one less but for residue 0
+            v[0][i] = rows[g * SH::RS + G::pad(INV ? ((res == 0 ? 0u : RM) - o) & RM : o)];
         }
+        __syncthreads();
+        W *yp = a.y + ((size_t)(tile / TPS) << L) + res;
+#pragma unroll
+        for (int i = 0; i < R; ++i)
+            yp[(size_t)(u0 + (uint32_t)i * (BLOCK / GPC)) << LC] = csub<W>(shoup<W>(v[0][i], a.c.ninv, a.c.ninvp, a.c.m), a.c.m);
     }
 }
 

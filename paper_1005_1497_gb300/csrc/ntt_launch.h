@@ -59,6 +59,10 @@ template <typename W> struct Launch {
     static cudaError_t rows_fwd(int L, const RowArgs<W> &a, int grid, cudaStream_t st);
     // rows of the twist form for transforms: whole trees of the row length in place
     static cudaError_t rows_uni(int L, const RowArgs<W> &a, int grid, cudaStream_t st);
+    // the same rows writing the natural order themselves, factor a.c.ninv:
+    // rows per tile (0: not for this length), and the launch over a.batch sequences
+    static int rows_out_rows(int L);
+    static cudaError_t rows_out(int L, bool inv, const NttArgs<W> &a, int grid, cudaStream_t st);
     static cudaError_t bitrev_out(int L, bool inv, const W *src, W *dst, long long batch, const ModC<W> &c,
                                   cudaStream_t st);
     // natural-order transform of whole sequences (L <= LRMAX)

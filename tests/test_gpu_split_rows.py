@@ -55,3 +55,23 @@ def test_word_aligned_pointers(ntt, m, L):
     orc = oracle.Oracle()
     idx = np.random.default_rng(L).integers(0, N, 24, dtype=np.uint64)
     assert np.array_equal(host(whole)[1][idx.astype(np.int64)], orc.conv_sample(host(f)[1], host(g)[1], m, idx))
+
+
+@pytest.mark.parametrize("m,L", [(M, 15), (M, 16), (M, 17), (M64, 14), (M64, 15)])
+def test_natural_order_from_rows(ntt, monkeypatch, m, L):
+    """Both sides of the tile limit above which the rows write the natural
+    order, and more tiles than the grid holds, against the row-twiddle form."""
+    N = 1 << L
+    monkeypatch.setenv("NTT_SPLIT_TWIST", "1")
+    twist = ntt.Plan(m, N)
+    monkeypatch.setenv("NTT_SPLIT_TWIST", "0")
+    rows = ntt.Plan(m, N)
+    gen = torch.Generator(device="cuda").manual_seed(90 + L)
+    for batch in (1, 2, 9, 40):
+        f = torch.randint(0, m, (batch, N), generator=gen, dtype=twist.dtype, device="cuda")
+        X = ntt.ntt_forward(rows, f)
+        assert torch.equal(ntt.ntt_forward(twist, f), X), batch
+        assert torch.equal(ntt.ntt_inverse(twist, X), f), batch
+        y = f.clone()
+        ntt.ntt_forward(twist, y, out=y)                      # in place
+        assert torch.equal(y, X), batch
