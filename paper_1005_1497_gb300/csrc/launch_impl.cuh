@@ -101,13 +101,15 @@ cudaError_t Launch<W>::conv_persistent(const PersistArgs<W> &a, int lmax, int gr
 }
 
 template <typename W, int L, class X>
-static cudaError_t launch_exact(const RowArgs<W> &a, const ExactArgs &e, int grid, cudaStream_t st)
+static cudaError_t launch_exact(const RowArgs<W> &a, const ExactFused &e, int grid, cudaStream_t st)
 {
     if constexpr (L <= LRMax<W>::v) {
-        const size_t smem = full_smem_of<W, L>();
-        static const cudaError_t init = ensure_smem(k_conv_exact<W, L, X>, smem);
+        constexpr int BLK = exact_block<W>(L);
+        constexpr size_t smem = L <= Arith<W>::RB + 5 ? FusedShape<W, L <= Arith<W>::RB + 5 ? L : 0, BLK>::smem
+                                                      : CRShape<W, L <= Arith<W>::RB + 5 ? LRMax<W>::v : L, true, L <= Arith<W>::RB + 5 ? BLOCK : BLK>::smem;
+        static const cudaError_t init = ensure_smem(k_conv_exact<W, L, X, BLK>, smem);
         if (init != cudaSuccess) return init;
-        k_conv_exact<W, L, X><<<grid, BLOCK, smem, st>>>(a, e);
+        k_conv_exact<W, L, X, BLK><<<grid, BLK, smem, st>>>(a, e);
         return launched();
     } else {
         return cudaErrorInvalidValue;
@@ -325,14 +327,14 @@ cudaError_t Launch<W>::conv_full(int L, int src, const RowArgs<W> &a, int grid, 
 }
 
 template <typename W>
-cudaError_t Launch<W>::conv_exact(int L, bool garner, const RowArgs<W> &a, const ExactArgs &e, int grid, cudaStream_t st)
+cudaError_t Launch<W>::conv_exact(int L, int primes, const RowArgs<W> &a, const ExactFused &e, int grid, cudaStream_t st)
 {
-    if (garner) {
-#define C(X) launch_exact<W, X, ExactGarner>(a, e, grid, st)
+    if (primes == 1) {
+#define C(X) launch_exact<W, X, ExactOne>(a, e, grid, st)
         NTT_SWITCH_L(C)
 #undef C
     }
-#define C(X) launch_exact<W, X, ExactResidues>(a, e, grid, st)
+#define C(X) launch_exact<W, X, ExactLast>(a, e, grid, st)
     NTT_SWITCH_L(C)
 #undef C
 }

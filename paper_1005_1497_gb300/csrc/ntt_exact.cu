@@ -25,6 +25,7 @@
 #include "ntt_internal.h"
 #include "nt_host.h"
 #include "ntt_count.h"
+#include "ntt_core.cuh"
 #include "ntt_exact.cuh"
 
 namespace {
@@ -276,7 +277,9 @@ struct ntt_exact_s {
     void **ptrs_g = nullptr;          // ptrs_f + KMAX
     void *host_ptrs[2 * KMAX] = {};   // the same pointers, host side
     int nsm = 0;
-    bool fused = false;               // whole sequences, 32-bit primes: residues and Garner fused into the convolutions
+    bool fused = false;               // one or two 32-bit primes, whole sequences: the ends fused into the convolutions
+    size_t fused_min = 0;             // from batches of this many pairs on
+    ntt::ExactFused last{};           // the fused launch's constants (the last prime's)
     bool all32 = false;               // every prime below 2^25: the 32-bit residue and reconstruction kernels
     Exact32 a32{};
 };
@@ -392,17 +395,34 @@ extern "C" ntt_status ntt_exact_plan(uint32_t N, uint32_t bound_bits, ntt_exact_
     int dev = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&e->nsm, cudaDevAttrMultiProcessorCount, dev);
-    // The fused form (NTT_EXACT_FUSED=1; whole sequences, 32-bit primes only)
-    // saves the residue and reconstruction passes' memory traffic, but adds
-    // their arithmetic to the IMAD-bound convolution kernels: measured 1.53
-    // against 0.98 ms for 8192 pairs of 2^12, so the three passes are the
-    // default.
-    const char *env = getenv("NTT_EXACT_FUSED");
-    e->fused = env && atoi(env) != 0;
-    for (int i = 0; i < e->k && e->fused; ++i) {
+    // The fused form (one or two 32-bit primes, whole sequences): one prime
+    // takes a single launch on the signed inputs, two fold the reconstruction
+    // into the second one's convolution.  Measured on GB300 against the
+    // separate passes (16.8 M elements, L = 11..14): one prime 194-211 ->
+    // 146-164 us, two primes 309-330 -> 289-304 us.  By default one prime from the batches
+    // on that do not run one block per pair, two for the column/row lengths;
+    // NTT_EXACT_FUSED=0|1 overrides.
+    if (e->all32 && e->k <= 2) {
         ntt_plan_info_t info;
-        ntt_plan_get_info(e->plans[i], &info);
-        if (info.word_bits != 32 || info.four_step) e->fused = false;
+        ntt_plan_get_info(e->plans[0], &info);
+        const bool row = info.log2N > (uint32_t)ntt::Arith<uint32_t>::RB + 5;
+        e->fused = !info.four_step && (e->k == 1 || row);
+        e->fused_min = e->k == 1 ? (size_t)info.small_max + 1 : 0;
+        if (const char *env = getenv("NTT_EXACT_FUSED")) {
+            e->fused = !info.four_step && atoi(env) != 0;
+            e->fused_min = 0;
+        }
+        const int i = e->k - 1;
+        const uint64_t m = a.p[i].m;
+        e->last.c = e->a32.c[i];
+        e->last.cp = e->a32.cp[i];
+        e->last.off = (uint32_t)(m - (1ull << 63) % m);
+        e->last.m0 = e->a32.m[0];
+        e->last.inv01 = e->a32.inv01;
+        e->last.inv01p = e->a32.inv01p;
+        e->last.M = e->a32.M;
+        e->last.half = e->a32.half;
+        e->last.prev = e->a32.rf[0];
     }
     *out = e;
     return NTT_OK;
@@ -438,22 +458,16 @@ extern "C" ntt_status conv_exact(ntt_exact_t e, const int64_t *f, const int64_t 
         const size_t off = p0 * e->N;
         const long long *fw = (const long long *)f + off, *gw = (const long long *)g + off;
         long long *hw = (long long *)h + off;
-        // scratch bases are 256-byte aligned and hold whole waves, so only the
-        // caller's bases decide the four-element path
-        if (e->fused) {
-            // one fused launch per prime: int64 inputs reduced in registers;
-            // the last prime reconstructs h from the others' residues
-            for (int i = 0; i < e->k; ++i) {
-                a.j = i;
-                a.h64 = hw;
-                for (int q = 0; q < KMAX; ++q) a.prev[q] = e->host_ptrs[q];
-                const bool last = i == e->k - 1;
-                ntt_status s = ntt_launch_exact(e->plans[i], last, fw, gw, last ? nullptr : e->host_ptrs[i], &a,
-                                                (long long)np, st);
-                if (s != NTT_OK) return s;
-            }
+        const bool fused = e->fused && np >= e->fused_min;
+        ntt::ExactFused last = e->last;
+        last.h64 = hw;
+        if (fused && e->k == 1) {
+            ntt_status s = ntt_launch_exact(e->plans[0], 1, fw, gw, &last, (long long)np, st);
+            if (s != NTT_OK) return s;
             continue;
         }
+        // scratch bases are 256-byte aligned and hold whole waves, so only the
+        // caller's bases decide the four-element path
         a.vec = ((((uintptr_t)fw | (uintptr_t)gw | (uintptr_t)hw) & 15u) == 0) ? 1 : 0;
         Exact32 b = e->a32;
         b.n = a.n;
@@ -471,9 +485,12 @@ extern "C" ntt_status conv_exact(ntt_exact_t e, const int64_t *f, const int64_t 
         cudaError_t err = ntt::launched();
         if (err != cudaSuccess) return ntt_fail(NTT_ERR_CUDA, "conv_exact: residues: %s", cudaGetErrorString(err));
         for (int i = 0; i < e->k; ++i) {
-            ntt_status s = conv_circular(e->plans[i], e->host_ptrs[i], e->host_ptrs[KMAX + i], e->host_ptrs[i], np, stream);
+            const bool fold = fused && i == e->k - 1;
+            ntt_status s = fold ? ntt_launch_exact(e->plans[i], 2, e->host_ptrs[i], e->host_ptrs[KMAX + i], &last, (long long)np, st)
+                                : conv_circular(e->plans[i], e->host_ptrs[i], e->host_ptrs[KMAX + i], e->host_ptrs[i], np, stream);
             if (s != NTT_OK) return s;
         }
+        if (fused) continue;
         if (fast && e->k == 1) k_exact_garner32<1><<<grid, threads, 0, st>>>(b, hw);
         else if (fast && e->k == 2) k_exact_garner32<2><<<grid, threads, 0, st>>>(b, hw);
         else k_exact_garner<<<grid, threads, 0, st>>>(a, e->ptrs_f, hw);

@@ -33,13 +33,6 @@ struct ExactArgs {
     uint64_t invp[XKMAX][XKMAX];    // floor(inv 2^64 / m_j)
     unsigned long long half_lo, half_hi;   // (M - 1) / 2
     unsigned long long M_lo, M_hi;         // M
-    // fused convolution kernels: the prime this launch reduces modulo, the
-    // earlier primes' residue arrays ([pairs][N], canonical) and, for the
-    // last prime, the signed 64-bit output ([pairs][N])
-    int j;
-    int pad;
-    const void *prev[XKMAX];
-    long long *h64;
 };
 
 __device__ __forceinline__ uint64_t shoup64(uint64_t b, uint64_t z, uint64_t zp, uint64_t m)
@@ -91,6 +84,49 @@ __device__ __forceinline__ long long garner(const ExactArgs &a, const uint64_t (
 __device__ __forceinline__ uint64_t load_res(const ExactArgs &a, const void *const *res, int j, long long i)
 {
     return a.p[j].word == 32 ? (uint64_t) static_cast<const uint32_t *>(res[j])[i] : static_cast<const uint64_t *>(res[j])[i];
+}
+
+// The ends of the exact convolution fused into one prime's convolution kernel
+// (one or two primes below 2^25; m and onep are the launch's ModC): signed
+// 64-bit inputs reduced in registers, and for the last prime the
+// reconstruction from its own residue and the first prime's.
+struct ExactFused {
+    uint32_t c, cp;                     // 2^32 mod m and its Shoup quotient
+    uint32_t off;                       // m - (2^63 mod m)
+    uint32_t m0;                        // two primes: the first,
+    uint32_t inv01, inv01p;             // its inverse mod m, and quotient
+    unsigned long long M, half;         // product of the primes and (M - 1) / 2
+    const uint32_t *prev;               // two primes: the first one's residues of h, [pairs][N]
+    long long *h64;                     // the output, [pairs][N]
+};
+
+// <x>_m of a signed 64-bit x.  x + 2^63 = hi 2^32 + lo; each half loses its
+// own multiple of m (Shoup, below 2m), and off takes 2^63 back: below 5m.
+__device__ __forceinline__ uint32_t residue_fused(long long x, const ExactFused &e, uint32_t m, uint32_t onep)
+{
+    const uint32_t lo = (uint32_t)(unsigned long long)x, hi = (uint32_t)((unsigned long long)x >> 32) ^ 0x80000000u;
+    const uint32_t q = __umulhi(hi, e.cp) + __umulhi(lo, onep);
+    uint32_t r = hi * e.c + (lo + e.off) - q * m;
+    r = min(r, r - 4 * m);
+    r = min(r, r - 2 * m);
+    return min(r, r - m);
+}
+
+// Garner for K = 1 or 2 primes, as in the reconstruction pass: v_0 = r_0,
+// v_1 = (r_1 - v_0) m_0^-1 mod m, X = v_0 + m_0 v_1 < M, signed in (-M/2, M/2].
+template <int K>
+__device__ __forceinline__ long long garner_fused(uint32_t r, uint32_t r0, const ExactFused &e, uint32_t m, uint32_t onep)
+{
+    unsigned long long X = r;
+    if constexpr (K == 2) {
+        uint32_t v = r0 - __umulhi(r0, onep) * m;
+        v = min(v, v - m);
+        const uint32_t d = r >= v ? r - v : r + m - v;
+        uint32_t v1 = d * e.inv01 - __umulhi(d, e.inv01p) * m;
+        v1 = min(v1, v1 - m);
+        X = r0 + (unsigned long long)v1 * e.m0;
+    }
+    return X > e.half ? (long long)(X - e.M) : (long long)X;
 }
 
 }  // namespace ntt

@@ -67,8 +67,9 @@ ntt_status ntt_launch_persistent(int word_bits, const void *descs, const void *i
                                  const ntt_plan_t *plans, int lmax, int grid, size_t smem, cudaStream_t st);   // plans: indexed by log2 N, null where absent
 size_t ntt_full_smem(int word_bits, int log2N);
 bool ntt_persist_class(int word_bits, int L);
-// the exact convolution's fused launch of one prime (32-bit plans of whole
-// sequences); exact_args: an ntt::ExactArgs
-ntt_status ntt_launch_exact(ntt_plan_t p, bool garner, const void *f64, const void *g64, void *h, const void *exact_args,
-                            long long np, cudaStream_t st);   // longest length a batch plan runs in its persistent launch
+// the exact convolution's fused launch (32-bit plans of whole sequences): one
+// prime from the signed 64-bit inputs f, g, or the second of two from its
+// residues f, g; exact_args: an ntt::ExactFused
+ntt_status ntt_launch_exact(ntt_plan_t p, int primes, const void *f, const void *g, const void *exact_args, long long np,
+                            cudaStream_t st);
 int ntt_num_sms();

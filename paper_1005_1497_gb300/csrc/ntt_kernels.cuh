@@ -112,18 +112,18 @@ __device__ __forceinline__ void stage_seq(const W *src, W *dst, uint32_t tau)
 
 // Input and output of the fused bodies: plain words (the default), or the
 // ends of the exact convolution fused in -- signed 64-bit inputs reduced
-// modulo the launch's prime (IN64), and for the last prime the Chinese
-// remainder reconstruction of each output from the earlier primes'
-// residues (GARNER), written as a signed 64-bit integer.
-struct NoExact { static constexpr bool IN64 = false, GARNER = false; };
-struct ExactResidues { static constexpr bool IN64 = true, GARNER = false; };
-struct ExactGarner { static constexpr bool IN64 = true, GARNER = true; };
+// modulo the launch's prime (IN64), and for the last of GARNER primes the
+// Chinese remainder reconstruction of each output, written as a signed
+// 64-bit integer.
+struct NoExact { static constexpr bool IN64 = false; static constexpr int GARNER = 0; };
+struct ExactOne { static constexpr bool IN64 = true; static constexpr int GARNER = 1; };
+struct ExactLast { static constexpr bool IN64 = false; static constexpr int GARNER = 2; };
 
 // Element i of a sequence whose first element is at base.
 template <class X, typename W>
-__device__ __forceinline__ W ld_elem(const W *base, uint32_t i, const ExactArgs *xa)
+__device__ __forceinline__ W ld_elem(const W *base, uint32_t i, const ExactFused *xa, const ModC<W> &c)
 {
-    if constexpr (X::IN64) return (W)residue(reinterpret_cast<const long long *>(base)[i], xa->p[xa->j]);
+    if constexpr (X::IN64) return (W)residue_fused(reinterpret_cast<const long long *>(base)[i], *xa, (uint32_t)c.m, (uint32_t)c.onep);
     else return base[i];
 }
 
@@ -137,19 +137,48 @@ __device__ __forceinline__ const W *seq_base(const W *batch, long long pair, uin
 
 // Canonical output r at index idx of sequence `pair` (hp: that sequence's words).
 template <class X, typename W>
-__device__ __forceinline__ void st_out(W *hp, long long pair, uint32_t N, uint32_t idx, W r, const ExactArgs *xa)
+__device__ __forceinline__ void st_out(W *hp, long long pair, uint32_t N, uint32_t idx, W r, const ExactFused *xa, const ModC<W> &c)
 {
-    if constexpr (X::GARNER) {
+    if constexpr (X::GARNER > 0) {
         const size_t at = (size_t)pair * N + idx;
-        uint64_t rr[XKMAX];
-#pragma unroll
-        for (int q = 0; q < XKMAX; ++q) {
-            if (q >= xa->k) break;
-            rr[q] = q == xa->j ? (uint64_t)r : load_res(*xa, xa->prev, q, (long long)at);
-        }
-        xa->h64[at] = garner(*xa, rr);
+        xa->h64[at] = garner_fused<X::GARNER>((uint32_t)r, X::GARNER == 2 ? xa->prev[at] : 0u, *xa, (uint32_t)c.m, (uint32_t)c.onep);
     } else {
         hp[idx] = r;
+    }
+}
+
+// VEC consecutive 64-bit inputs reduced, and VEC consecutive outputs
+// reconstructed (idx a multiple of VEC), two per access where aligned.
+template <int VEC, typename W>
+__device__ __forceinline__ void ld_residues(const long long *p, W (&d)[VEC], bool wide, const ExactFused *xa, const ModC<W> &c)
+{
+    long long x[VEC];
+    if (wide && VEC > 1) {
+#pragma unroll
+        for (int e = 0; e < VEC; e += 2) {
+            const longlong2 q = *reinterpret_cast<const longlong2 *>(p + e);
+            x[e] = q.x; x[e + 1] = q.y;
+        }
+    } else {
+#pragma unroll
+        for (int e = 0; e < VEC; ++e) x[e] = p[e];
+    }
+#pragma unroll
+    for (int e = 0; e < VEC; ++e) d[e] = (W)residue_fused(x[e], *xa, (uint32_t)c.m, (uint32_t)c.onep);
+}
+
+template <int K, int VEC, typename W>
+__device__ __forceinline__ void st_garner(size_t at, const W (&r)[VEC], const W *r0, bool wide, const ExactFused *xa, const ModC<W> &c)
+{
+    long long h[VEC];
+#pragma unroll
+    for (int e = 0; e < VEC; ++e) h[e] = garner_fused<K>((uint32_t)r[e], K == 2 ? (uint32_t)r0[e] : 0u, *xa, (uint32_t)c.m, (uint32_t)c.onep);
+    if (wide && VEC > 1) {
+#pragma unroll
+        for (int e = 0; e < VEC; e += 2) *reinterpret_cast<longlong2 *>(xa->h64 + at + e) = make_longlong2(h[e], h[e + 1]);
+    } else {
+#pragma unroll
+        for (int e = 0; e < VEC; ++e) xa->h64[at + e] = h[e];
     }
 }
 
@@ -165,7 +194,7 @@ __device__ __forceinline__ void st_out(W *hp, long long pair, uint32_t N, uint32
 // Rows [base + group, a.nrows) by steps of stride.
 template <typename W, int L, int SRC, class X = NoExact, int BLK = BLOCK>
 __device__ __forceinline__ void conv_fused_body(const RowArgs<W> &a, long long base, long long stride,
-                                                const ExactArgs *xa = nullptr)
+                                                const ExactFused *xa = nullptr)
 {
     using G = Geo<W, L>;
     using SH = FusedShape<W, L, BLK>;
@@ -226,8 +255,8 @@ __device__ __forceinline__ void conv_fused_body(const RowArgs<W> &a, long long b
                 v[0][k] = B[x];
                 v[1][k] = S[BG::ROWP + x];
             } else {
-                v[0][k] = ld_elem<X>(fp, x, xa);
-                v[1][k] = ld_elem<X>(gp, x, xa);
+                v[0][k] = ld_elem<X>(fp, x, xa, a.c);
+                v[1][k] = ld_elem<X>(gp, x, xa, a.c);
             }
         }
         if constexpr (STAGE) {
@@ -249,7 +278,7 @@ __device__ __forceinline__ void conv_fused_body(const RowArgs<W> &a, long long b
 #pragma unroll
             for (int k = 0; k < R; ++k) {
                 const uint32_t x = b0 + ((uint32_t)k << lo0);
-                st_out<X>(hp, a.pair0 + rho, N, block_out<L>(x), canon<W>(v[0][k], a.c.cB, a.c.cBp, a.c.m), xa);
+                st_out<X>(hp, a.pair0 + rho, N, block_out<L>(x), canon<W>(v[0][k], a.c.cB, a.c.cBp, a.c.m), xa, a.c);
             }
         } else {                                            // one thread per pair, no exchange
             fwd_all<W, L, L, 0, 2, TW_SMEM, true>(v, 0u, tau, S, gid, stw, a.c);
@@ -258,7 +287,7 @@ __device__ __forceinline__ void conv_fused_body(const RowArgs<W> &a, long long b
             dit_all<W, L, last, TW_SMEM>(v[0], 0u, tau, S, gid, stw, a.c);
 #pragma unroll
             for (int k = 0; k < R; ++k)
-                st_out<X>(hp, a.pair0 + rho, N, (N - (uint32_t)k) & (N - 1u), canon<W>(v[0][k], (W)1, a.c.onep, a.c.m), xa);
+                st_out<X>(hp, a.pair0 + rho, N, (N - (uint32_t)k) & (N - 1u), canon<W>(v[0][k], (W)1, a.c.onep, a.c.m), xa, a.c);
         }
     }
 }
@@ -465,7 +494,7 @@ __device__ __forceinline__ void cols_from_rows(const W *S, uint32_t stride, uint
 // factor 2^(B + BB) / N is in the twist's diagonal.
 template <typename W, int L, int SRC, bool ITEM = false, int OUT = 0, class X = NoExact, int BLK = BLOCK>
 __device__ __forceinline__ void conv_cr_body(const RowArgs<W> &a, long long base, long long stride, long long end = 0,
-                                             const ExactArgs *xa = nullptr)
+                                             const ExactFused *xa = nullptr)
 {
     using SH = CRShape<W, L, true, BLK>;
     constexpr int RW = SH::RW, LC = SH::LC, RC = SH::RC, TPP = SH::TPP, PPC = SH::PPC, CPT = SH::CPT, VEC = SH::VEC;
@@ -515,8 +544,7 @@ __device__ __forceinline__ void conv_cr_body(const RowArgs<W> &a, long long base
                     const uint32_t x = col_of(j) + ((uint32_t)k << RW);
                     W t[VEC];
                     if constexpr (X::IN64) {
-#pragma unroll
-                        for (int e = 0; e < VEC; ++e) t[e] = ld_elem<X>(src, x + e, xa);
+                        ld_residues<VEC>(reinterpret_cast<const long long *>(src) + x, t, wide, xa, a.c);
                     } else {
                         ld_vec<W, VEC>(src + x, t, wide);
                     }
@@ -524,7 +552,7 @@ __device__ __forceinline__ void conv_cr_body(const RowArgs<W> &a, long long base
                     for (int e = 0; e < VEC; ++e) dst[(j * VEC + e) * RC + k] = t[e];
                 }
         };
-        if (!X::IN64 && VEC > 1 && ((uintptr_t)src & (VEC * sizeof(W) - 1)) == 0) all(true);
+        if (VEC > 1 && ((uintptr_t)src & (X::IN64 ? 15u : VEC * sizeof(W) - 1)) == 0) all(true);
         else all(false);
     };
     auto store_cols = [&](const W (&v)[R], W *S) {          // into the rows' slices
@@ -618,10 +646,23 @@ __device__ __forceinline__ void conv_cr_body(const RowArgs<W> &a, long long base
         if constexpr (STAGE) cp_async_wait();
         psync();
         // inverse, column phase
+        W r0[X::GARNER == 2 ? R : 1];                       // the first prime's residues of this thread's outputs
+        if constexpr (X::GARNER == 2) {
+            const uint32_t *prev = xa->prev + (size_t)(a.pair0 + (live ? rho : base)) * N;
+#pragma unroll
+            for (int j = 0; j < CPT / VEC; ++j)
+#pragma unroll
+                for (int k = 0; k < RC; ++k) {
+                    uint32_t t[VEC];                        // (the plan's scratch: aligned)
+                    ld_vec<uint32_t, VEC>(prev + block_out<L>(col_of(j) + ((uint32_t)k << RW)), t, true);
+#pragma unroll
+                    for (int e = 0; e < VEC; ++e) r0[(j * RC + k) * VEC + e] = t[e];
+                }
+        }
         cols_from_rows<W, RW, LC, VEC, TPP, true>(P, 2 * GR::ROWP, ptau, v[0]);
         bcold_all<W, LC, RW, VEC, TPP, 0, CPT / VEC, R>(v[0], ptau, stw, a.c);
         if (!live) continue;                                // (no barrier follows in this round)
-        const bool wide = ((uintptr_t)hcur & (VEC * sizeof(W) - 1)) == 0;
+        const bool wide = X::GARNER > 0 ? ((uintptr_t)xa->h64 & 15u) == 0 : ((uintptr_t)hcur & (VEC * sizeof(W) - 1)) == 0;
 #pragma unroll
         for (int j = 0; j < CPT / VEC; ++j)
 #pragma unroll
@@ -635,9 +676,8 @@ __device__ __forceinline__ void conv_cr_body(const RowArgs<W> &a, long long base
                 } else {
 #pragma unroll
                     for (int e = 0; e < VEC; ++e) t[e] = canon<W>(t[e], a.c.cB, a.c.cBp, a.c.m);
-                    if constexpr (X::GARNER) {
-#pragma unroll
-                        for (int e = 0; e < VEC; ++e) st_out<X>(hcur, a.pair0 + rho, N, block_out<L>(x + e), t[e], xa);
+                    if constexpr (X::GARNER > 0) {
+                        st_garner<X::GARNER, VEC>((size_t)(a.pair0 + rho) * N + block_out<L>(x), t, r0 + (X::GARNER == 2 ? (j * RC + k) * VEC : 0), wide, xa, a.c);
                     } else {
                         st_vec<W, VEC>(hcur + block_out<L>(x), t, wide);
                     }
@@ -737,20 +777,25 @@ __global__ void __launch_bounds__(BLOCK, 1) k_conv_rows(const __grid_constant__ 
     }
 }
 
-// The exact convolution's fused launches (whole sequences, contiguous):
-// X = ExactResidues for every prime but the last (its residues of h go to
-// a.h), X = ExactGarner for the last (h goes to e.h64 as signed integers).
-template <typename W, int L, class X>
-__global__ void __launch_bounds__(BLOCK, 1) k_conv_exact(const __grid_constant__ RowArgs<W> a,
-                                                          const __grid_constant__ ExactArgs e)
+// The exact convolution's fused launches (whole sequences, contiguous; h goes
+// to e.h64 as signed integers).  X = ExactOne: the whole convolution of a
+// plan of one prime, 24 bytes per element instead of 48.  X = ExactLast: the
+// second of two primes from its residues, reconstructing from its own and
+// the first one's result, 60 bytes instead of 72; reading the inputs in both
+// primes' kernels (48 bytes) measured 321 us against 303 at 4096 x 2^12
+// (separate passes 318), since 64-bit inputs leave no shared memory to stage
+// them in.
+template <typename W, int L, class X, int BLK>
+__global__ void __launch_bounds__(BLK, BLOCK / BLK) k_conv_exact(const __grid_constant__ RowArgs<W> a,
+                                                                const __grid_constant__ ExactFused e)
 {
     constexpr int RW = Arith<W>::RB + 5;
     if constexpr (L <= RW) {
-        constexpr int GPC = FusedShape<W, L>::GPC;
-        conv_fused_body<W, L, 0, X>(a, (long long)blockIdx.x * GPC, (long long)gridDim.x * GPC, &e);
+        constexpr int GPC = FusedShape<W, L, BLK>::GPC;
+        conv_fused_body<W, L, 0, X, BLK>(a, (long long)blockIdx.x * GPC, (long long)gridDim.x * GPC, &e);
     } else {
-        constexpr int PPC = CRShape<W, L, true>::PPC;
-        conv_cr_body<W, L, 0, false, 0, X>(a, (long long)blockIdx.x * PPC, (long long)gridDim.x * PPC, 0, &e);
+        constexpr int PPC = CRShape<W, L, true, BLK>::PPC;
+        conv_cr_body<W, L, 0, false, 0, X, BLK>(a, (long long)blockIdx.x * PPC, (long long)gridDim.x * PPC, 0, &e);
     }
 }
 

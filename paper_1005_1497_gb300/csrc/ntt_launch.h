@@ -31,6 +31,10 @@ template <typename W> constexpr int split_row_bits(int L, bool twisted)
 // Threads per block of the twist form's row kernel.
 template <typename W> constexpr int row_block(int LR) { return LR < LRMax<W>::v ? BLOCK_HALF : BLOCK; }
 
+// Threads per block of the exact convolution's fused kernels: half blocks for
+// the column/row lengths below the longest, as for plain convolutions.
+template <typename W> constexpr int exact_block(int L) { return L > Arith<W>::RB + 5 && L < LRMax<W>::v ? BLOCK_HALF : BLOCK; }
+
 template <typename W> struct Launch {
     static constexpr int LRMAX = LRMax<W>::v;
     static constexpr int LMAX = 20;            // split path: LMAX - LRMAX column bits, in two passes above 5
@@ -72,10 +76,10 @@ template <typename W> struct Launch {
                              const ModC<W> &c, int grid, cudaStream_t st);
     static cudaError_t check_range(const W *data, long long n, W m, unsigned long long *bad, int grid,
                                    cudaStream_t st);
-    // the exact convolution's fused launch of one prime (whole sequences,
-    // contiguous, signed 64-bit inputs): residues of h to a.h, or (garner)
-    // the reconstructed signed 64-bit h to e.h64
-    static cudaError_t conv_exact(int L, bool garner, const RowArgs<W> &a, const ExactArgs &e, int grid, cudaStream_t st);
+    // the exact convolution's fused launch (whole sequences, contiguous,
+    // signed 64-bit h to e.h64): a plan of one prime from its signed 64-bit
+    // inputs, or the second of two primes from its residues
+    static cudaError_t conv_exact(int L, int primes, const RowArgs<W> &a, const ExactFused &e, int grid, cudaStream_t st);
     // dynamic shared memory of the whole-sequence fused kernel of length 2^L
     static size_t conv_full_smem(int L);
     // one persistent launch over a work list of whole-sequence items
