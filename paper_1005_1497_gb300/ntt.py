@@ -118,12 +118,17 @@ def launch_count() -> int:
     return int(lib().ntt_launch_count())
 
 
-def _stream(stream) -> ctypes.c_void_p:
+def _stream(stream) -> int:
+    """The cudaStream_t of `stream` (default: torch's current stream of the
+    current device, read as a raw handle: a Stream object costs more than the
+    launch of a short convolution)."""
     if stream is None:
-        stream = torch.cuda.current_stream()
+        if not torch.cuda.is_initialized():
+            torch.cuda.init()
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
     if isinstance(stream, torch.cuda.Stream):
-        return ctypes.c_void_p(stream.cuda_stream)
-    return ctypes.c_void_p(int(stream))
+        return stream.cuda_stream
+    return int(stream)
 
 
 _DT = {32: (torch.int32, torch.uint32), 64: (torch.int64, torch.uint64)}
@@ -145,6 +150,7 @@ class Plan:
         self.block = int(info.block)
         self.small_max = int(info.small_max)   # batches up to this run one block per pair
         self.dtype = _DT[self.word_bits][0]
+        self._dtypes = _DT[self.word_bits]
 
     def close(self):
         if getattr(self, "handle", None) and self.handle.value:
@@ -159,6 +165,10 @@ class Plan:
 
     def check(self, t: torch.Tensor, name: str) -> int:
         """Validate a buffer of whole sequences; return its batch size."""
+        if t.is_cuda and t.dtype in self._dtypes and t.is_contiguous():
+            n = t.numel()
+            if n and not n % self.N:
+                return n // self.N
         if not t.is_cuda:
             raise ValueError(f"{name} must be a CUDA tensor")
         if t.dtype not in _DT[self.word_bits]:
@@ -179,17 +189,25 @@ def ntt_plan(m: int, N: int) -> Plan:
 
 def ntt_forward(plan: Plan, x: torch.Tensor, out: torch.Tensor | None = None, stream=None) -> torch.Tensor:
     b = plan.check(x, "x")
-    out = torch.empty_like(x) if out is None else out
-    plan.check(out, "out")
-    _check(lib().ntt_forward(plan.handle, x.data_ptr(), out.data_ptr(), b, _stream(stream)), "ntt_forward")
+    if out is None:
+        out = torch.empty_like(x)
+    else:
+        plan.check(out, "out")
+    st = lib().ntt_forward(plan.handle, x.data_ptr(), out.data_ptr(), b, _stream(stream))
+    if st:
+        _check(st, "ntt_forward")
     return out
 
 
 def ntt_inverse(plan: Plan, X: torch.Tensor, out: torch.Tensor | None = None, stream=None) -> torch.Tensor:
     b = plan.check(X, "X")
-    out = torch.empty_like(X) if out is None else out
-    plan.check(out, "out")
-    _check(lib().ntt_inverse(plan.handle, X.data_ptr(), out.data_ptr(), b, _stream(stream)), "ntt_inverse")
+    if out is None:
+        out = torch.empty_like(X)
+    else:
+        plan.check(out, "out")
+    st = lib().ntt_inverse(plan.handle, X.data_ptr(), out.data_ptr(), b, _stream(stream))
+    if st:
+        _check(st, "ntt_inverse")
     return out
 
 
@@ -198,10 +216,13 @@ def conv_circular(plan: Plan, f: torch.Tensor, g: torch.Tensor, out: torch.Tenso
     b = plan.check(f, "f")
     if plan.check(g, "g") != b:
         raise ValueError("f and g hold different numbers of sequences")
-    out = torch.empty_like(f) if out is None else out
-    plan.check(out, "out")
-    _check(lib().conv_circular(plan.handle, f.data_ptr(), g.data_ptr(), out.data_ptr(), b, _stream(stream)),
-           "conv_circular")
+    if out is None:
+        out = torch.empty_like(f)
+    else:
+        plan.check(out, "out")
+    st = lib().conv_circular(plan.handle, f.data_ptr(), g.data_ptr(), out.data_ptr(), b, _stream(stream))
+    if st:
+        _check(st, "conv_circular")
     return out
 
 
