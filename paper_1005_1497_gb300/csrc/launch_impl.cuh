@@ -139,6 +139,8 @@ static cudaError_t launch_conv_rows(bool twisted, const RowArgs<W> &a, int grid,
             static const cudaError_t init = ensure_smem(k_conv_cr<W, LR, 0, 1, BLK>, smem);
             if (init != cudaSuccess) return init;
             k_conv_cr<W, LR, 0, 1, BLK><<<grid, BLK, smem, st>>>(a);
+        } else if constexpr (std::is_same<W, r64>::value) {
+            return cudaErrorInvalidValue;                   // (the row-twiddle form reads the plan's table as it is)
         } else {
             constexpr int LR = LRMax<W>::v;
             constexpr size_t smem = CRShape<W, LR, false>::smem;

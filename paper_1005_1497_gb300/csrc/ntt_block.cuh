@@ -35,6 +35,9 @@
 // levels with unit butterflies, 2m more for each of the other ten: at most
 // 112m, below the word.  The last factor 2^BB N^{-1} 2^B (Shoup) takes any
 // word and brings N'^{-1} and Montgomery's 2^B.
+// Roomy 64-bit moduli (r64, m < 2^48; N <= 2^13): products below 13m, so 8m +
+// 8 13m = 112m forward, T < 4 112^2 m^2 < 2^112, Montgomery's result below
+// 2m, and 71m + 9 13m < 2^8 m < 2^56 inverse.
 #pragma once
 
 #include "ntt_core.cuh"
@@ -49,6 +52,7 @@ constexpr int BLOCK_LMIN = BB + 1;
 template <typename W> struct Wide;
 template <> struct Wide<uint32_t> { using T = uint64_t; };
 template <> struct Wide<uint64_t> { using T = unsigned __int128; };
+template <> struct Wide<r64> { using T = unsigned __int128; };
 
 __device__ __forceinline__ uint32_t mont(uint64_t T, const ModC<uint32_t> &c)
 {
@@ -56,10 +60,11 @@ __device__ __forceinline__ uint32_t mont(uint64_t T, const ModC<uint32_t> &c)
     return (uint32_t)((T + (uint64_t)q * c.m) >> 32);
 }
 
-__device__ __forceinline__ uint64_t mont(unsigned __int128 T, const ModC<uint64_t> &c)
+template <typename W>
+__device__ __forceinline__ W mont(unsigned __int128 T, const ModC<W> &c)
 {
-    const uint64_t lo = (uint64_t)T, q = lo * c.mneg;
-    return (uint64_t)(T >> 64) + __umul64hi(q, c.m) + (lo != 0ull ? 1ull : 0ull);
+    const W lo = (W)T, q = lo * c.mneg;
+    return (W)(T >> 64) + __umul64hi(q, c.m) + (lo != 0 ? 1 : 0);
 }
 
 // Shared-memory rows of the block form.  32-bit words with rows of at least

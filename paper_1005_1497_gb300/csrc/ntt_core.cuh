@@ -38,6 +38,7 @@
 #pragma once
 
 #include <cstdint>
+#include <type_traits>
 #include <cuda_runtime.h>
 
 namespace ntt {
@@ -57,6 +58,18 @@ template <> struct Arith<uint64_t> {
     static constexpr int PADSH = 4;     // one pad word per 16 eight-byte words
     __device__ __forceinline__ static uint64_t mulhi(uint64_t a, uint64_t b) { return __umul64hi(a, b); }
 };
+
+// 64-bit words of moduli below 2^ROOMY_BITS, as a type of their own (the same
+// size and values as uint64_t): the lazy bounds have 2^16 and more to spare
+// there, so a product may take its quotient from three partial products
+// instead of four, two bits short, and leave a value below 13m.  Kernels on
+// this type read the twiddle table staged with its quotients shifted by two
+// (floor(z 2^62 / m)); ModC::m2 holds 13m, the multiple of m above any product.
+using r64 = unsigned long long;
+static_assert(!std::is_same<r64, uint64_t>::value && sizeof(r64) == sizeof(uint64_t), "a distinct 64-bit type");
+constexpr int ROOMY_BITS = 48, ROOMY_M2 = 13;
+
+template <> struct Arith<r64> : Arith<uint64_t> {};
 
 // Per-plan constants, passed by value in the kernel parameters.
 template <typename W> struct ModC {
@@ -91,6 +104,49 @@ __device__ __forceinline__ uint32_t shoup<uint32_t>(uint32_t b, uint32_t z, uint
     asm("mul.hi.u32 %0, %1, %2;" : "=r"(q) : "r"(b), "r"(zp));
     asm("mul.lo.u32 %0, %1, %2;" : "=r"(t) : "r"(b), "r"(z));
     asm("mad.lo.u32 %0, %1, %2, %3;" : "=r"(r) : "r"(q), "r"(0u - m), "r"(t));
+    return r;
+}
+
+// A product below 2m whatever the word type, from the full quotient.
+template <typename W>
+__device__ __forceinline__ W shoup_full(W b, W z, W zp, W m)
+{
+    if constexpr (std::is_same<W, r64>::value) return (W)shoup<uint64_t>((uint64_t)b, (uint64_t)z, (uint64_t)zp, (uint64_t)m);
+    else return shoup<W>(b, z, zp, m);
+}
+
+// Roomy moduli: p = floor(z 2^62 / m), b < 2^56.  The quotient 4 (b1 p1 +
+// hi(b1 p0) + hi(b0 p1)) misses b z / m by less than 12 + 2^-6 (two floors and
+// the product b0 p0, each below one unit of 4), so the result lies in [0,
+// 13m).  Three high products and a low one for it, six multiply-adds for b z
+// - 4 q m: 28 multiply-pipe cycles and about 10 instructions against 32 and 19.
+template <>
+__device__ __forceinline__ r64 shoup<r64>(r64 b, r64 z, r64 p, r64 m)
+{
+    const r64 n = 0ull - 4ull * m;
+    r64 r;
+    asm("{\n\t"
+        ".reg .u32 b0, b1, z0, z1, p0, p1, n0, n1, q0, q1, t, lo, hi;\n\t"
+        ".reg .u64 q, w;\n\t"
+        "mov.b64 {b0, b1}, %1;\n\t"
+        "mov.b64 {z0, z1}, %2;\n\t"
+        "mov.b64 {p0, p1}, %3;\n\t"
+        "mov.b64 {n0, n1}, %4;\n\t"
+        "mul.hi.u32 t, b0, p1;\n\t"
+        "mad.hi.u32 t, b1, p0, t;\n\t"
+        "cvt.u64.u32 w, t;\n\t"
+        "mad.wide.u32 q, b1, p1, w;\n\t"
+        "mov.b64 {q0, q1}, q;\n\t"
+        "mul.wide.u32 w, b0, z0;\n\t"
+        "mad.wide.u32 w, q0, n0, w;\n\t"
+        "mov.b64 {lo, hi}, w;\n\t"
+        "mad.lo.u32 hi, b0, z1, hi;\n\t"
+        "mad.lo.u32 hi, b1, z0, hi;\n\t"
+        "mad.lo.u32 hi, q0, n1, hi;\n\t"
+        "mad.lo.u32 hi, q1, n0, hi;\n\t"
+        "mov.b64 %0, {lo, hi};\n\t"
+        "}"
+        : "=l"(r) : "l"(b), "l"(z), "l"(p), "l"(n));
     return r;
 }
 
@@ -165,14 +221,17 @@ __device__ __forceinline__ uint32_t pointwise(uint32_t F, uint32_t G, const ModC
     return hi + __umulhi(q, c.m) + (lo != 0u ? 1u : 0u);
 }
 
-__device__ __forceinline__ uint64_t pointwise(uint64_t F, uint64_t G, const ModC<uint64_t> &c)
+template <typename W>
+__device__ __forceinline__ W pointwise64(W F, W G, const ModC<W> &c)
 {
-    uint64_t u = shoup<uint64_t>(F, c.cN, c.cNp, c.m);
-    uint64_t lo = u * G;
-    uint64_t hi = __umul64hi(u, G);
-    uint64_t q = lo * c.mneg;
-    return hi + __umul64hi(q, c.m) + (lo != 0ull ? 1ull : 0ull);
+    W u = shoup_full<W>(F, c.cN, c.cNp, c.m);
+    W lo = u * G;
+    W hi = __umul64hi(u, G);
+    W q = lo * c.mneg;
+    return hi + __umul64hi(q, c.m) + (lo != 0 ? 1 : 0);
 }
+__device__ __forceinline__ uint64_t pointwise(uint64_t F, uint64_t G, const ModC<uint64_t> &c) { return pointwise64<uint64_t>(F, G, c); }
+__device__ __forceinline__ r64 pointwise(r64 F, r64 G, const ModC<r64> &c) { return pointwise64<r64>(F, G, c); }
 
 // ---------------------------------------------------------------- geometry
 
@@ -281,7 +340,11 @@ __device__ __forceinline__ void stage_twiddles(const W *__restrict__ tw, W *stw,
     constexpr int PC = tw_per_chunk<W>();
     const uint32_t chunks = (pairs + PC - 1) / PC;
     for (uint32_t c = threadIdx.x; c < chunks; c += blockDim.x) {
-        if (PC == 2 && pairs == 1) {
+        if constexpr (std::is_same<W, r64>::value) {
+            ulonglong2 q = __ldg(reinterpret_cast<const ulonglong2 *>(tw) + c);
+            q.y >>= 2;                                      // (see r64)
+            reinterpret_cast<ulonglong2 *>(stw)[tw_swz(c)] = q;
+        } else if (PC == 2 && pairs == 1) {
             reinterpret_cast<uint2 *>(stw)[0] = __ldg(reinterpret_cast<const uint2 *>(tw));
         } else {
             reinterpret_cast<uint4 *>(stw)[tw_swz(c)] = __ldg(reinterpret_cast<const uint4 *>(tw) + c);
@@ -598,6 +661,6 @@ __device__ __forceinline__ void gather_natural(W (&v)[Geo<W, L>::R], const W *S,
 // Final canonical residue of a lazily bounded value: Shoup product by the
 // factor (z, zp) (1 or N^-1) into [0, 2m), then one conditional subtraction.
 template <typename W>
-__device__ __forceinline__ W canon(W v, W z, W zp, W m) { return csub<W>(shoup<W>(v, z, zp, m), m); }
+__device__ __forceinline__ W canon(W v, W z, W zp, W m) { return csub<W>(shoup_full<W>(v, z, zp, m), m); }
 
 }  // namespace ntt

@@ -20,6 +20,7 @@ constexpr int BLOCK_HALF = 256;
 template <typename W> struct LRMax;        // longest row one block transforms
 template <> struct LRMax<uint32_t> { static constexpr int v = 14; };
 template <> struct LRMax<uint64_t> { static constexpr int v = 13; };
+template <> struct LRMax<r64> { static constexpr int v = 13; };
 
 // One convolution of an uneven batch, as seen by the device.
 template <typename W> struct DevDesc {
