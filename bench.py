@@ -604,7 +604,7 @@ def measure_uniform(name, args, world, rank, local, sub=False):
         ems = max_over_ranks(world, (time.perf_counter() - t0) * 1000.0 / esteps)
         out["e2e"] = {"value": round(pairs_total * 1000.0 / ems, 1), "unit": "conv/s", "ms_per_step": round(ems, 3),
                       "h2d_bytes_per_step": 2 * batch * N * wb, "d2h_bytes_per_step": batch * N * wb,
-                      "entry": ("conv_circular_host (pinned host buffers: " + ("read and written in place by the kernel" if 3 * batch * N * wb <= (96 << 20) and not plan.four_step else "chunked copy/compute overlap") + ")"),
+                      "entry": ("conv_circular_host (pinned host buffers: " + ("read and written in place by the kernel" if 3 * batch * N * wb <= ((320 if wb == 4 and N >= 1024 else 96) << 20) and not plan.four_step else "chunked copy/compute overlap") + ")"),
                       "bit_identical_to_device_path": bool(torch.equal(hh, h.cpu()))}
         # the host link alone, for the same bytes (plain copies, untimed
         # above): f and g in, h out, and both directions at once -- the

@@ -168,7 +168,8 @@ ntt_status conv_circular_plain(ntt_plan_t plan, const void *f_dev, const void *g
  * staging memory (4 slots x 3 chunks, about 300 MB at most) is allocated on
  * first use and kept by the plan.  With page-locked buffers (cudaHostAlloc /
  * cudaHostRegister), which the GPU can address over the C2C link, and
- * whole-sequence lengths, a batch whose f, g and h total at most 96 MB is
+ * whole-sequence lengths, a batch whose f, g and h total at most 96 MB
+ * (320 MB for 32-bit words from 2^10 on) is
  * instead read and written in place by the kernels (no copies: lower latency
  * for small batches; larger batches are faster through the copy pipeline).
  * The environment variable NTT_HOST_DIRECT=p (0..100) overrides that choice

@@ -28,7 +28,9 @@ template <typename W, int L, int SRC, int BLK>
 static cudaError_t launch_conv_full_blk(const RowArgs<W> &a, int grid, cudaStream_t st)
 {
     constexpr int RW = Arith<W>::RB + 5;
-    if constexpr (L <= RW) {
+    if constexpr (SRC == 2 && L < HOST_LMIN) {
+        return cudaErrorInvalidValue;
+    } else if constexpr (L <= RW) {
         constexpr size_t smem = FusedShape<W, L, BLK>::smem;
         static const cudaError_t init = ensure_smem(k_conv_fused<W, L, SRC, BLK>, smem);
         if (init != cudaSuccess) return init;
@@ -325,6 +327,8 @@ template <typename W>
 cudaError_t Launch<W>::conv_full(int L, int src, const RowArgs<W> &a, int grid, cudaStream_t st, int block)
 {
     if (!block_ok(L, block)) return cudaErrorInvalidValue;
+    if constexpr (sizeof(W) == 4)
+        if (src == 2) return conv_full_src<2>(L, a, grid, st, block);
     return src == 1 ? conv_full_src<1>(L, a, grid, st, block) : conv_full_src<0>(L, a, grid, st, block);
 }
 

@@ -352,7 +352,7 @@ static cudaError_t launch_rows(ntt_plan_t p, bool twisted, const RowArgs<W> &a, 
 template <typename W>
 static cudaError_t conv_dispatch(ntt_plan_t p, const W *f, const W *g, W *h, const DevDesc<W> *descs,
                                  long long pair0, long long batch, W *scratch, uint32_t wave, cudaStream_t st,
-                                 int twist = -1)
+                                 int twist = -1, bool host = false)
 {
     const bool tw_form = twist < 0 ? p->twist : twist != 0;
     const ModC<W> &c = modc<W>(p);
@@ -363,7 +363,7 @@ static cudaError_t conv_dispatch(ntt_plan_t p, const W *f, const W *g, W *h, con
         if (mode == 0 && batch <= p->small_max)
             return Launch<W>::conv_small(p->L, a, (int)std::min<long long>(batch, (long long)p->nsm * Launch<W>::SMALL_PER_SM), st);
         const int grid = row_grid(p->nsm, batch, Launch<W>::pairs_per_block(p->L, p->block), ntt::BLOCK / p->block);
-        return launch_full<W>(p, mode, a, grid, st);
+        return launch_full<W>(p, host && sizeof(W) == 4 && p->L >= ntt::HOST_LMIN ? 2 : mode, a, grid, st);
     }
     const long long N = p->N;
     for (long long w0 = 0; w0 < batch; w0 += wave) {
@@ -453,18 +453,23 @@ extern "C" ntt_status ntt_inverse(ntt_plan_t p, const void *X, void *x, size_t b
     return e == cudaSuccess ? NTT_OK : cuda_fail(e, "ntt_inverse");
 }
 
+// conv_circular; `host`: the buffers are page-locked host memory.
+static ntt_status conv_contiguous(ntt_plan_t p, const void *f, const void *g, void *h, size_t batch, cudaStream_t st, bool host)
+{
+    cudaError_t e = p->word == 32
+        ? conv_dispatch<uint32_t>(p, (const uint32_t *)f, (const uint32_t *)g, (uint32_t *)h, nullptr, 0,
+                                  (long long)batch, (uint32_t *)p->scratch, p->wave, st, -1, host)
+        : conv_dispatch<uint64_t>(p, (const uint64_t *)f, (const uint64_t *)g, (uint64_t *)h, nullptr, 0,
+                                  (long long)batch, (uint64_t *)p->scratch, p->wave, st, -1, host);
+    return e == cudaSuccess ? NTT_OK : cuda_fail(e, "conv_circular");
+}
+
 extern "C" ntt_status conv_circular(ntt_plan_t p, const void *f, const void *g, void *h, size_t batch,
                                     ntt_stream_t stream)
 {
     ntt::Trace tr("conv_circular");
     if (!p || !f || !g || !h || batch == 0) return ntt_fail(NTT_ERR_ARG, "conv_circular: invalid argument");
-    cudaStream_t st = (cudaStream_t)stream;
-    cudaError_t e = p->word == 32
-        ? conv_dispatch<uint32_t>(p, (const uint32_t *)f, (const uint32_t *)g, (uint32_t *)h, nullptr, 0,
-                                  (long long)batch, (uint32_t *)p->scratch, p->wave, st)
-        : conv_dispatch<uint64_t>(p, (const uint64_t *)f, (const uint64_t *)g, (uint64_t *)h, nullptr, 0,
-                                  (long long)batch, (uint64_t *)p->scratch, p->wave, st);
-    return e == cudaSuccess ? NTT_OK : cuda_fail(e, "conv_circular");
+    return conv_contiguous(p, f, g, h, batch, (cudaStream_t)stream, false);
 }
 
 extern "C" ntt_status conv_circular_plain(ntt_plan_t p, const void *f, const void *g, void *h, size_t batch,
@@ -521,23 +526,25 @@ extern "C" ntt_status conv_circular_host(ntt_plan_t p, const void *f, const void
     const size_t seq = (size_t)p->N * elt;
     // Page-locked buffers can also be read and written in place by the
     // kernels over the C2C link.  By default a batch whose inputs and output
-    // total at most DIRECT_MAX bytes goes that way whole (no copies to wait
-    // for: measured on GB300, 1 x 2^10 end to end 33 -> 19 us, 256 x 2^14
-    // 0.31 -> 0.25 ms; from about 192 MB on the staged copies are faster,
-    // 1024 x 2^14 0.876 against 0.892 ms).  NTT_HOST_DIRECT (percent)
-    // overrides that: its share of the pairs goes in place on its own stream
-    // while the copy engines stage the rest.
-    constexpr size_t DIRECT_MAX = (size_t)96 << 20;
+    // total at most `direct_max` bytes goes that way whole (no copies to wait
+    // for).  Measured on GB300, in place against the copies: 1 x 2^10 18
+    // against 33 us, 256 x 2^14 (48 MB) 227 against 309, 1024 x 2^14 (192 MB)
+    // 796 against 866, 1500 x 2^14 (281 MB) 1150 against 1247, from 384 MB on
+    // within 3%; the shorter lengths, whose kernels stage, 16384 x 2^8 (48 MB)
+    // 263 against 296 but 65536 x 2^8 (192 MB) 1052 against 854.
+    // NTT_HOST_DIRECT (percent) overrides that: its share of the pairs goes in
+    // place on its own stream while the copy engines stage the rest.
+    const size_t direct_max = (size_t)(p->word == 32 && p->L >= ntt::HOST_LMIN ? 320 : 96) << 20;
     size_t ndirect = 0;
     const void *fd = host_device_address(f), *gd = host_device_address(g);
     void *hd = const_cast<void *>(host_device_address(h));
     if (fd && gd && hd && !p->split) {
         const char *env = getenv("NTT_HOST_DIRECT");
-        const int pct = env ? std::max(0, std::min(100, atoi(env))) : (3 * batch * seq <= DIRECT_MAX ? 100 : 0);
+        const int pct = env ? std::max(0, std::min(100, atoi(env))) : (3 * batch * seq <= direct_max ? 100 : 0);
         ndirect = batch * (size_t)pct / 100;
     }
     if (ndirect == batch) {
-        ntt_status s = conv_circular(p, fd, gd, hd, batch, stream);
+        ntt_status s = conv_contiguous(p, fd, gd, hd, batch, (cudaStream_t)stream, true);
         if (s != NTT_OK) return s;
         CUDA_TRY(cudaStreamSynchronize((cudaStream_t)stream), "conv_circular_host: sync");
         return NTT_OK;
@@ -573,7 +580,7 @@ extern "C" ntt_status conv_circular_host(ntt_plan_t p, const void *f, const void
     for (cudaStream_t st : p->hstream) CUDA_TRY(cudaStreamWaitEvent(st, start, 0), "wait");
     cudaEventDestroy(start);
     if (ndirect) {                                  // the in-place share, on the user stream
-        ntt_status s = conv_circular(p, fd, gd, hd, ndirect, stream);
+        ntt_status s = conv_contiguous(p, fd, gd, hd, ndirect, (cudaStream_t)stream, true);
         if (s != NTT_OK) return s;
     }
     const unsigned char *fb = (const unsigned char *)f, *gb = (const unsigned char *)g;

@@ -30,8 +30,8 @@ template <typename W> struct DevDesc {
 };
 
 // Arguments of the row kernels.  For a whole-sequence launch (L == LR) row
-// rho is pair pair0 + rho of the batch (contiguous arrays f, g, h or the
-// descriptor list).  For the split path (L > LR) rho counts rows of the
+// rho is pair pair0 + rho of the batch: SRC 0 contiguous arrays f, g, h, SRC 1
+// the descriptor list, SRC 2 contiguous arrays in page-locked host memory.  For the split path (L > LR) rho counts rows of the
 // current wave inside the scratch arrays f (= F~, overwritten by H~) and g.
 template <typename W> struct RowArgs {
     const W *f;
@@ -223,7 +223,7 @@ __device__ __forceinline__ void conv_fused_body(const RowArgs<W> &a, long long b
         }
     };
     constexpr uint32_t INB = X::IN64 ? 8u : (uint32_t)sizeof(W);     // bytes per input element
-    constexpr bool STAGE = SH::STAGE && !X::IN64;
+    constexpr bool STAGE = SH::STAGE && !X::IN64 && SRC != 2;
     W *B = reinterpret_cast<W *>(smem_raw + SH::next) + (size_t)gid * N;
     using BG = BGeo<W, L>;
     const W *fp, *gp, *fn = nullptr, *gn = nullptr;
@@ -504,7 +504,7 @@ __device__ __forceinline__ void conv_cr_body(const RowArgs<W> &a, long long base
     static_assert(LC >= 1 && CPT * RC == R, "column/row split");
     constexpr uint32_t N = 1u << L;
     constexpr int last = GR::NPASS - 1;
-    constexpr bool STAGE = SH::STAGE && !X::IN64;
+    constexpr bool STAGE = SH::STAGE && !X::IN64 && SRC != 2;
     constexpr uint32_t INB = X::IN64 ? 8u : (uint32_t)sizeof(W);     // bytes per input element
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int pid = threadIdx.x / TPP;
@@ -576,7 +576,9 @@ __device__ __forceinline__ void conv_cr_body(const RowArgs<W> &a, long long base
     // measured on GB300, 4096 x 2^14 412 -> 394 us at equal clocks (without
     // any global load: 369), 8192 x 2^13 392 -> 376, 2^12 1.5%, 2^11 equal.
     // 64-bit words, whose padded rows take 8-byte copies only, lose by it
-    // (301 x 2^13: 59.4 -> 61.5 us); there the next f is loaded into registers
+    // (301 x 2^13: 59.4 -> 61.5 us), and so do inputs in host memory (SRC 2),
+    // whose copies all SMs would issue and wait for at the same time (256 x
+    // 2^14 over C2C 254 -> 301 us); there the next f is loaded into registers
     // after the block products, and g while f's columns are transformed.
     W *G = reinterpret_cast<W *>(smem_raw + SH::tw_bytes + SH::rows_bytes) + ((size_t)pid << L);
     auto stage_f = [&](const W *f) { stage_row<W, RW, true>(f + ((size_t)wr << RW), Srow + GR::ROWP, lane); };

@@ -8,6 +8,7 @@
 
 namespace ntt {
 
+constexpr int HOST_LMIN = 10;                  // lengths whose kernels read host memory without staging it
 constexpr int CMAX = 5;                        // column bits of one pass of the split path
 
 // log2 of the split path's row length (L > LRMax).  The column passes are
@@ -45,7 +46,8 @@ template <typename W> struct Launch {
     static int pairs_per_block(int L, int block = BLOCK);
     // whether the whole-sequence fused kernels of length 2^L come with `block` threads
     static bool block_ok(int L, int block);
-    // whole-sequence fused convolution (L <= LRMAX); src 0 = contiguous, 1 = descriptors
+    // whole-sequence fused convolution (L <= LRMAX); src 0 = contiguous, 1 = descriptors,
+    // 2 = contiguous in host memory (32-bit words, L >= HOST_LMIN)
     static cudaError_t conv_full(int L, int src, const RowArgs<W> &a, int grid, cudaStream_t st, int block = BLOCK);
     // (one source mode; instantiated in separate translation units)
     template <int SRC>
