@@ -53,7 +53,7 @@ struct BatchClass {
     ntt_plan_t plan = nullptr;       // cached, not owned
     size_t off = 0;                  // first descriptor of the class in the device list
     size_t count = 0;
-    void *scratch = nullptr;         // split path: owned by the batch plan
+    void *scratch = nullptr;         // split path: its stream's, shared by the classes there
     uint32_t wave = 0;
     double work = 0;                 // N log N count: classes launch largest work first
     int stream = 0;
@@ -75,6 +75,7 @@ struct ntt_batch_s {
     size_t count = 0;
     std::vector<cudaStream_t> streams;
     std::vector<cudaEvent_t> done;
+    std::vector<void *> scratch;     // per stream
     cudaEvent_t fork = nullptr;
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t gexec = nullptr;
@@ -87,7 +88,7 @@ extern "C" void ntt_batch_destroy(ntt_batch_t b)
     if (!b) return;
     if (b->gexec) cudaGraphExecDestroy(b->gexec);
     if (b->graph) cudaGraphDestroy(b->graph);
-    for (auto &c : b->classes) cudaFree(c.scratch);
+    for (void *p : b->scratch) cudaFree(p);
     cudaFree(b->descs);
     cudaFree(b->items);
     cudaFree(b->counter);
@@ -143,17 +144,6 @@ extern "C" ntt_status ntt_batch_plan(uint64_t m, const ntt_conv_desc *descs, siz
     if (cudaMemcpy(b->descs, host.data(), host.size(), cudaMemcpyHostToDevice) != cudaSuccess)
         return bail(ntt_fail(NTT_ERR_CUDA, "ntt_batch_plan: upload descriptors"));
 
-    // split classes get their own scratch so that classes run concurrently
-    for (auto &c : b->classes) {
-        ntt_plan_info_t info;
-        ntt_plan_get_info(c.plan, &info);
-        if (info.four_step) {
-            c.wave = std::min<uint32_t>(info.wave, (uint32_t)c.count);
-            if (!ntt::dev_alloc(&c.scratch, 2 * (size_t)c.wave * ((size_t)1 << c.L) * elt))
-                return bail(ntt_fail(NTT_ERR_OOM, "ntt_batch_plan: scratch"));
-        }
-    }
-
     // Short lengths become work items of a single persistent launch on
     // stream 0; each item covers two rounds of a block's rows in flight.
     // Longer lengths keep their own launches (stream assignment below).
@@ -181,17 +171,60 @@ extern "C" ntt_status ntt_batch_plan(uint64_t m, const ntt_conv_desc *descs, siz
             return bail(ntt_fail(NTT_ERR_CUDA, "ntt_batch_plan: upload work list"));
         b->persist_grid = std::min(ntt_num_sms(), b->nitems);
     }
-    // Streams: the persistent launch on one, every class with launches of its
-    // own on another, one after the other, largest work first.  Each of those
-    // classes' kernels fills the GPU, so running two at once only makes them
-    // interfere: measured on GB300 (10,000 uneven pairs, graph replay) 7.80 ms
-    // with them spread over three streams by longest processing time, 7.44 ms
-    // on one beside the persistent launch's, 7.47 ms with everything on one.
+    // Streams: the persistent launch on the first; on the second, one after
+    // the other and largest work first, the classes whose kernels fill the
+    // GPU, as running two of those at once only makes them interfere (measured
+    // on GB300, 10,000 uneven pairs by graph replay: 7.80 ms with them spread
+    // over three streams by longest processing time, 7.44 ms on one).  A class
+    // of at most one round of blocks leaves SMs idle and costs that round's
+    // latency however few its pairs are: such classes are dealt to the second
+    // and a third stream by the rounds they take (100 uneven pairs of 2^6 ..
+    // 2^19, every class below a round: 187 us on two streams, 134 on three;
+    // 2000 pairs 1388 and 1375; 400 of 2^15 .. 2^17, classes of 3 to 5 rounds
+    // all on the second stream: 296 and 294).
     if (nsplit == 0 && b->nitems == 0) return bail(ntt_fail(NTT_ERR_ARG, "ntt_batch_plan: empty batch"));
-    const int K = (b->nitems && nsplit) ? 2 : 1;
-    const int own = K - 1;                                   // stream of the own-launch classes
+    const int own = b->nitems ? 1 : 0;                       // first stream of the own-launch classes
+    const double round = (double)((size_t)ntt_num_sms() << lrmax);   // elements of one round
+    auto elements = [](const BatchClass &c) { return (double)c.count * (double)((size_t)1 << c.L); };
+    double load[2] = {0, 0};
     for (auto &c : b->classes)
-        if (c.stream != -1) c.stream = own;
+        if (c.stream != -1 && elements(c) > round) {
+            c.stream = own;
+            load[0] += elements(c) / round;
+        }
+    for (auto &c : b->classes)
+        if (c.stream != -1 && elements(c) <= round) {
+            const int k = load[1] < load[0];
+            c.stream = own + k;
+            load[k] += 1;
+        }
+    const int K = own + (load[0] > 0) + (load[1] > 0);
+    // Scratch of the split classes, as the plans' own may be in use elsewhere:
+    // one piece per stream, used by its classes in turn, for every pair of a
+    // class in one wave up to SCRATCH_MAX (fewer, fuller launches: measured on
+    // GB300, 143 x 2^19 in waves of 64 pairs 721 us, in one 679 us), for the
+    // plan's own wave at least, and that where memory is short.
+    constexpr size_t SCRATCH_MAX = (size_t)1 << 30;
+    b->scratch.assign(K, nullptr);
+    for (int k = 0; k < K; ++k)
+        for (size_t limit = SCRATCH_MAX;; limit = 0) {
+            size_t bytes = 0;
+            for (auto &c : b->classes) {
+                ntt_plan_info_t info;
+                ntt_plan_get_info(c.plan, &info);
+                if (c.stream != k || !info.four_step) continue;
+                const size_t per_pair = 2 * ((size_t)1 << c.L) * elt;
+                c.wave = (uint32_t)std::min<size_t>(std::max<size_t>(info.wave, limit / per_pair), c.count);
+                bytes = std::max(bytes, c.wave * per_pair);
+            }
+            if (bytes == 0) break;
+            if (ntt::dev_alloc(&b->scratch[k], bytes)) {
+                for (auto &c : b->classes)
+                    if (c.stream == k) c.scratch = b->scratch[k];
+                break;
+            }
+            if (limit == 0) return bail(ntt_fail(NTT_ERR_OOM, "ntt_batch_plan: scratch"));
+        }
     b->streams.resize(K);
     b->done.resize(K);
     for (int i = 0; i < K; ++i) {
