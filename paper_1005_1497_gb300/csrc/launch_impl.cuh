@@ -308,7 +308,7 @@ static cudaError_t launch_conv_small(const RowArgs<W> &a, int grid, cudaStream_t
         constexpr size_t smem = SmallShape<W, L>::smem;
         static const cudaError_t init = ensure_smem(k_conv_small<W, L>, smem);
         if (init != cudaSuccess) return init;
-        k_conv_small<W, L><<<grid, SMALL_THREADS, smem, st>>>(a);
+        k_conv_small<W, L><<<grid, SmallShape<W, L>::THREADS, smem, st>>>(a);
         return launched();
     } else {
         return cudaErrorInvalidValue;

@@ -146,13 +146,28 @@ __device__ __forceinline__ void bfwd_all(W (&v)[2][Geo<W, LR>::R], uint32_t rowo
     }
 }
 
+// The four elements from v[0][b] on <- their product with those from v[1][b]
+// on modulo x^4 - z, or x^4 + z (plus), times 2^-B.
+template <typename W, int R>
+__device__ __forceinline__ void block_product(W (&v)[2][R], const int b, const bool plus, W z, W zp, const ModC<W> &c)
+{
+    using D = typename Wide<W>::T;
+    const W f0 = v[0][b], f1 = v[0][b + 1], f2 = v[0][b + 2], f3 = v[0][b + 3];
+    const W g0 = v[1][b], g1 = v[1][b + 1], g2 = v[1][b + 2], g3 = v[1][b + 3];
+    W y1 = shoup<W>(g1, z, zp, c.m), y2 = shoup<W>(g2, z, zp, c.m), y3 = shoup<W>(g3, z, zp, c.m);
+    if (plus) { y1 = c.m2 - y1; y2 = c.m2 - y2; y3 = c.m2 - y3; }
+    v[0][b] = mont((D)f0 * g0 + (D)f1 * y3 + (D)f2 * y2 + (D)f3 * y1, c);
+    v[0][b + 1] = mont((D)f0 * g1 + (D)f1 * g0 + (D)f2 * y3 + (D)f3 * y2, c);
+    v[0][b + 2] = mont((D)f0 * g2 + (D)f1 * g1 + (D)f2 * g0 + (D)f3 * y3, c);
+    v[0][b + 3] = mont((D)f0 * g3 + (D)f1 * g2 + (D)f2 * g1 + (D)f3 * g0, c);
+}
+
 // v[0] <- v[0] v[1] modulo the factors of the thread's R consecutive
 // elements (first at index xbase): blocks 2i and 2i + 1 modulo x^4 - z_i and
 // x^4 + z_i, times 2^-B.
 template <typename W, int R>
 __device__ __forceinline__ void block_products(W (&v)[2][R], uint32_t xbase, const W *__restrict__ tw, const ModC<W> &c)
 {
-    using D = typename Wide<W>::T;
     constexpr int CNT = R >> (BB + 1);
     constexpr int CH = (CNT >= 2 && tw_per_chunk<W>() == 2) ? 2 : 1;
     const uint32_t nb = xbase >> (BB + 1);
@@ -164,16 +179,7 @@ __device__ __forceinline__ void block_products(W (&v)[2][R], uint32_t xbase, con
         for (int tt = 0; tt < CH; ++tt)
 #pragma unroll
             for (int s = 0; s < 2; ++s) {
-                const int b = ((t0 + tt) << (BB + 1)) + (s << BB);
-                const W f0 = v[0][b], f1 = v[0][b + 1], f2 = v[0][b + 2], f3 = v[0][b + 3];
-                const W g0 = v[1][b], g1 = v[1][b + 1], g2 = v[1][b + 2], g3 = v[1][b + 3];
-                W y1 = shoup<W>(g1, z[tt], zp[tt], c.m), y2 = shoup<W>(g2, z[tt], zp[tt], c.m),
-                  y3 = shoup<W>(g3, z[tt], zp[tt], c.m);
-                if (s == 1) { y1 = c.m2 - y1; y2 = c.m2 - y2; y3 = c.m2 - y3; }
-                v[0][b] = mont((D)f0 * g0 + (D)f1 * y3 + (D)f2 * y2 + (D)f3 * y1, c);
-                v[0][b + 1] = mont((D)f0 * g1 + (D)f1 * g0 + (D)f2 * y3 + (D)f3 * y2, c);
-                v[0][b + 2] = mont((D)f0 * g2 + (D)f1 * g1 + (D)f2 * g0 + (D)f3 * y3, c);
-                v[0][b + 3] = mont((D)f0 * g3 + (D)f1 * g2 + (D)f2 * g1 + (D)f3 * g0, c);
+                block_product<W, R>(v, ((t0 + tt) << (BB + 1)) + (s << BB), s == 1, z[tt], zp[tt], c);
             }
     }
 }

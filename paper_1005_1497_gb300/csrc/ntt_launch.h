@@ -55,7 +55,7 @@ template <typename W> struct Launch {
     // one pair per block (k_conv_small) for the one-warp lengths (L <= RB + 5),
     // contiguous pairs; grid blocks walk the pairs
     static cudaError_t conv_small(int L, const RowArgs<W> &a, int grid, cudaStream_t st);
-    static constexpr int SMALL_PER_SM = 8;     // blocks of k_conv_small resident per SM (256 threads, <= 37 registers)
+    static constexpr int SMALL_PER_SM = 32;    // largest grid of k_conv_small per SM (blocks of 32 to 256 threads)
     // split path pieces (LRMAX < L <= LMAX); cols_fwd / cols_inv run one or
     // two column passes
     // (twisted: the four-step twist form, see the twist in ntt_kernels.cuh)
