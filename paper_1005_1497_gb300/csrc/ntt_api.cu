@@ -319,10 +319,12 @@ static int row_grid(int nsm, long long rows, int per_block, int per_sm = 1)
 
 // The fused kernels' launches; 64-bit words of roomy moduli on their own type
 // (see r64 in ntt_core.cuh).  Measured on GB300 against the general 64-bit
-// kernels: 301 x 2^13 59.4 -> 53.3 us, 12 x 2^17 74.4 -> 64.3 us, bit-identical.
-template <typename W> static RowArgs<ntt::r64> as_roomy(const RowArgs<W> &a)
+// kernels: 301 x 2^13 59.4 -> 53.3 us, 12 x 2^17 74.4 -> 64.3 us; natural-order
+// transforms 2048 x 2^12 71.3 -> 58.7, 1024 x 2^13 80.3 -> 72.3, 64 x 2^17 122
+// -> 114 us; bit-identical.
+template <template <typename> class Args, typename W> static Args<ntt::r64> as_roomy(const Args<W> &a)
 {
-    RowArgs<ntt::r64> r;
+    Args<ntt::r64> r;
     static_assert(sizeof r == sizeof a && sizeof(W) == sizeof(ntt::r64), "the same layout");
     memcpy(&r, &a, sizeof r);
     r.c.m2 = ntt::ROOMY_M2 * r.c.m;
@@ -389,9 +391,14 @@ static cudaError_t ntt_dispatch(ntt_plan_t p, const W *x, W *y, long long batch,
 {
     const ModC<W> &c = modc<W>(p);
     const W *tw = (const W *)p->tw;
+    [[maybe_unused]] const bool roomy = p->m < (1ull << ntt::ROOMY_BITS);
     if (!p->split) {
         NttArgs<W> a{x, y, batch, tw, c};
-        return Launch<W>::ntt_full(p->L, inv, a, row_grid(p->nsm, batch, Launch<W>::rows_per_block(p->L)), st);
+        const int grid = row_grid(p->nsm, batch, Launch<W>::rows_per_block(p->L));
+        if constexpr (sizeof(W) == 8) {
+            if (roomy) return Launch<ntt::r64>::ntt_full(p->L, inv, as_roomy(a), grid, st);
+        }
+        return Launch<W>::ntt_full(p->L, inv, a, grid, st);
     }
     const long long N = p->N;
     W *scratch = (W *)p->scratch;
@@ -419,13 +426,23 @@ static cudaError_t ntt_dispatch(ntt_plan_t p, const W *x, W *y, long long batch,
         const int per = twisted ? Launch<W>::rows_out_rows(p->L) : 0;
         if (per && rows / per >= 32) {
             NttArgs<W> na{scratch, y + (size_t)w0 * N, np, tw, cs};
-            e = Launch<W>::rows_out(p->L, inv, na, (int)std::min<long long>(rows / per, p->nsm), st);
+            const int grid = (int)std::min<long long>(rows / per, p->nsm);
+            if constexpr (sizeof(W) == 8) {
+                e = roomy ? Launch<ntt::r64>::rows_out(p->L, inv, as_roomy(na), grid, st) : Launch<W>::rows_out(p->L, inv, na, grid, st);
+            } else {
+                e = Launch<W>::rows_out(p->L, inv, na, grid, st);
+            }
             if (e != cudaSuccess) return e;
             continue;
         }
         RowArgs<W> ra{scratch, nullptr, nullptr, nullptr, rows, 0, tw, c};
         const int grid = row_grid(p->nsm, rows, Launch<W>::rows_per_block(lr));
-        e = twisted ? Launch<W>::rows_uni(p->L, ra, grid, st) : Launch<W>::rows_fwd(p->L, ra, grid, st);
+        if constexpr (sizeof(W) == 8) {
+            if (twisted && roomy) e = Launch<ntt::r64>::rows_uni(p->L, as_roomy(ra), grid, st);
+            else e = twisted ? Launch<W>::rows_uni(p->L, ra, grid, st) : Launch<W>::rows_fwd(p->L, ra, grid, st);
+        } else {
+            e = twisted ? Launch<W>::rows_uni(p->L, ra, grid, st) : Launch<W>::rows_fwd(p->L, ra, grid, st);
+        }
         if (e != cudaSuccess) return e;
         e = Launch<W>::bitrev_out(p->L, inv, scratch, y + (size_t)w0 * N, np, cs, st);
         if (e != cudaSuccess) return e;

@@ -357,7 +357,8 @@ __device__ __forceinline__ void stage_twiddles(const W *__restrict__ tw, W *stw,
 // sequence), so node 0 has the twiddle 1.  Bound note: inputs < m, level 0
 // leaves < 2m and every node-0 butterfly of levels 1..4 doubles the bound
 // (< 2^(d+1) m after level d), the others add 2m: at most 32m + 2m (L - 5)
-// after the forward, below 50m for L <= 14.
+// after the forward, below 50m for L <= 14 (r64: 32m + 13m (L - 5), below
+// 2^8 m < 2^56 for L <= 13).
 // UN: the last level whose node 0 skips the product.
 template <typename W, int L, int LR, int P, int JJ, int NS, int TWS, bool Z0 = false, int UN = 4>
 __device__ __forceinline__ void fwd_level(W (&v)[NS][Geo<W, LR>::R], uint32_t xbase,

@@ -950,7 +950,7 @@ __global__ void __launch_bounds__(BLOCK, 1) k_ntt_rows(const __grid_constant__ N
         W *yp = a.y + (size_t)rho * N;
 #pragma unroll
         for (int k = 0; k < R; ++k)
-            yp[b0 + ((uint32_t)k << G::lo(0))] = csub<W>(INV ? shoup<W>(v[0][k], a.c.ninv, a.c.ninvp, a.c.m)
+            yp[b0 + ((uint32_t)k << G::lo(0))] = csub<W>(INV ? shoup_full<W>(v[0][k], a.c.ninv, a.c.ninvp, a.c.m)
                                                              : shoup_one<W>(v[0][k], a.c.onep, a.c.m), a.c.m);
     }
 }
@@ -1422,7 +1422,7 @@ __global__ void __launch_bounds__(BLOCK, 1) k_rows_out(const __grid_constant__ N
         W *yp = a.y + ((size_t)(tile / TPS) << L) + res;
 #pragma unroll
         for (int i = 0; i < R; ++i)
-            yp[(size_t)(u0 + (uint32_t)i * (BLOCK / GPC)) << LC] = csub<W>(shoup<W>(v[0][i], a.c.ninv, a.c.ninvp, a.c.m), a.c.m);
+            yp[(size_t)(u0 + (uint32_t)i * (BLOCK / GPC)) << LC] = canon<W>(v[0][i], a.c.ninv, a.c.ninvp, a.c.m);
     }
 }
 
