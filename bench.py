@@ -509,11 +509,11 @@ def measure_uniform(name, args, world, rank, local, sub=False):
     hbm_ach = alg_bytes / (ms * 1e-3) / 1e9
     if plan.four_step:
         kernel_tag = None
-        kernel = ("split path, per wave k_cols_fwd + k_conv_cr<u32,14,14,0,1> (rows: 2^(L-14) whole length-2^14 "
-                  "convolutions per pair, the dominant kernel) + k_cols_inv")
+        kernel = ("split path, per wave k_cols_fwd + k_conv_cr<.,LR,0,1> (rows: 2^(L-LR) whole length-2^LR "
+                  "convolutions per pair, LR <= 14, the dominant kernel) + k_cols_inv")
     elif L > (9 if args.m64 else 10):
         kernel_tag = None if args.m64 else f"k_conv_cr_u32_L{L}_{batch}x{N}"
-        kernel = f"k_conv_cr<u{8 * wb},{L},{L},0,0,{plan.block}> (fused, column/row form)"
+        kernel = f"k_conv_cr<u{8 * wb},{L},0,0,{plan.block}> (fused, column/row form)"
     elif batch <= plan.small_max:
         kernel_tag = None
         kernel = f"k_conv_small<u{8 * wb},{L}> (fused, one thread block per pair: a batch too small to fill the GPU)"
@@ -902,7 +902,7 @@ def measure_uneven(args, world, rank, local, sub=False):
            "roofline": {"bound": "alu", "achieved": round(alu_ach, 1), "peak": round(alu_peak, 1),
                         "unit": "Gmodmul/s", "frac": round(alu_ach / alu_peak, 4), "traffic": None,
                         "kernel": "all length classes of one step (graph replay); the split classes' rows "
-                                  "(k_conv_cr<u32,14,14,·,1>) dominate"},
+                                  "(k_conv_cr<u32,LR,·,1>) dominate"},
            "roofline_hbm": {"bound": "hbm", "achieved": round(alg_bytes / (ms * 1e-3) / 1e9, 1), "peak": hbm_peak,
                             "unit": "GB/s", "frac": round(alg_bytes / (ms * 1e-3) / 1e9 / hbm_peak, 4),
                             "peak_src": f"{peak_src} copy bandwidth"},
