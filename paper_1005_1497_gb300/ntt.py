@@ -134,6 +134,24 @@ def _stream(stream) -> int:
 _DT = {32: (torch.int32, torch.uint32), 64: (torch.int64, torch.uint64)}
 
 
+def _check_room(t: torch.Tensor, name: str, nbytes: int):
+    """A buffer that the kernels write `nbytes` bytes to: memory the GPU can
+    reach (its own, or page-locked), contiguous, large enough."""
+    if not (t.is_cuda or t.is_pinned()):
+        raise ValueError(f"{name} must be a CUDA tensor")
+    if not t.is_contiguous():
+        raise ValueError(f"{name} must be contiguous")
+    if t.numel() * t.element_size() < nbytes:
+        raise ValueError(f"{name}: {t.numel() * t.element_size()} bytes, {nbytes} needed")
+
+
+def _check_out(t: torch.Tensor, words: int, word_bits: int):
+    """An output of `words` words; only the word size of its dtype counts."""
+    if t.element_size() * 8 != word_bits:
+        raise TypeError(f"out: dtype {t.dtype} does not match {word_bits}-bit words")
+    _check_room(t, "out", words * word_bits // 8)
+
+
 class Plan:
     """``ntt_plan(m, N)``: validated parameters and resident twiddle table."""
 
@@ -179,6 +197,12 @@ class Plan:
             raise ValueError(f"{name}: {t.numel()} words is not a whole number of length-{self.N} sequences")
         return t.numel() // self.N
 
+    def check_out(self, t: torch.Tensor, batch: int):
+        """Validate an output of `batch` sequences (room for more is fine)."""
+        n = self.check(t, "out")
+        if n < batch:
+            raise ValueError(f"out holds {n} sequences, {batch} are written")
+
     def empty(self, batch: int, device="cuda") -> torch.Tensor:
         return torch.empty((batch, self.N), dtype=self.dtype, device=device)
 
@@ -192,7 +216,7 @@ def ntt_forward(plan: Plan, x: torch.Tensor, out: torch.Tensor | None = None, st
     if out is None:
         out = torch.empty_like(x)
     else:
-        plan.check(out, "out")
+        plan.check_out(out, b)
     st = lib().ntt_forward(plan.handle, x.data_ptr(), out.data_ptr(), b, _stream(stream))
     if st:
         _check(st, "ntt_forward")
@@ -204,7 +228,7 @@ def ntt_inverse(plan: Plan, X: torch.Tensor, out: torch.Tensor | None = None, st
     if out is None:
         out = torch.empty_like(X)
     else:
-        plan.check(out, "out")
+        plan.check_out(out, b)
     st = lib().ntt_inverse(plan.handle, X.data_ptr(), out.data_ptr(), b, _stream(stream))
     if st:
         _check(st, "ntt_inverse")
@@ -219,7 +243,7 @@ def conv_circular(plan: Plan, f: torch.Tensor, g: torch.Tensor, out: torch.Tenso
     if out is None:
         out = torch.empty_like(f)
     else:
-        plan.check(out, "out")
+        plan.check_out(out, b)
     st = lib().conv_circular(plan.handle, f.data_ptr(), g.data_ptr(), out.data_ptr(), b, _stream(stream))
     if st:
         _check(st, "conv_circular")
@@ -231,10 +255,16 @@ def conv_circular_plain(plan: Plan, f: torch.Tensor, g: torch.Tensor, out: torch
     b = plan.check(f, "f")
     if plan.check(g, "g") != b:
         raise ValueError("f and g hold different numbers of sequences")
-    out = torch.empty_like(f) if out is None else out
-    work = torch.empty((2 * b, plan.N), dtype=f.dtype, device=f.device) if work is None else work
-    if work.numel() < 2 * b * plan.N:
+    if out is None:
+        out = torch.empty_like(f)
+    else:
+        _check_out(out, b * plan.N, plan.word_bits)
+    if work is None:
+        work = torch.empty((2 * b, plan.N), dtype=f.dtype, device=f.device)
+    elif work.numel() < 2 * b * plan.N:
         raise ValueError("work must hold 2 * batch * N words")
+    else:
+        _check_room(work, "work", 2 * b * plan.N * plan.word_bits // 8)
     _check(lib().conv_circular_plain(plan.handle, f.data_ptr(), g.data_ptr(), out.data_ptr(), b, work.data_ptr(),
                                      _stream(stream)), "conv_circular_plain")
     return out
@@ -305,9 +335,12 @@ def conv_exact(plan: ExactPlan, f: torch.Tensor, g: torch.Tensor, out: torch.Ten
             raise ValueError(f"{name} has length {t.shape[-1]}, the plan N={plan.N}")
     if f.shape != g.shape:
         raise ValueError("f and g must have the same shape")
-    out = torch.empty_like(f) if out is None else out
-    if out.shape != f.shape or out.dtype != torch.int64 or not out.is_contiguous():
+    if out is None:
+        out = torch.empty_like(f)
+    elif out.shape != f.shape or out.dtype != torch.int64:
         raise ValueError("out must be a contiguous int64 tensor shaped like f")
+    else:
+        _check_out(out, f.numel(), 64)
     b = f.numel() // plan.N
     _check(lib().conv_exact(plan.handle, f.data_ptr(), g.data_ptr(), out.data_ptr(), b, _stream(stream)),
            "conv_exact")
@@ -327,7 +360,10 @@ def conv_circular_shift(m: int, f: torch.Tensor, g: torch.Tensor, out: torch.Ten
             raise ValueError(f"{name} must be a contiguous 32-bit CUDA tensor")
     if f.shape != g.shape:
         raise ValueError("f and g must have the same shape")
-    out = torch.empty_like(f) if out is None else out
+    if out is None:
+        out = torch.empty_like(f)
+    else:
+        _check_out(out, f.numel(), 32)
     N = f.shape[-1]
     b = f.numel() // N
     _check(lib().conv_circular_shift(m, N, f.data_ptr(), g.data_ptr(), out.data_ptr(), b, mode, _stream(stream)),
