@@ -371,14 +371,22 @@ def conv_circular_shift(m: int, f: torch.Tensor, g: torch.Tensor, out: torch.Ten
     return out
 
 
-def _descs(triples):
+def _word_bytes(m: int) -> int:
+    """Bytes per word of the buffers modulo m (32-bit words below 2^25)."""
+    return 4 if m < 1 << 25 else 8
+
+
+def _descs(m, triples):
     arr = (ConvDesc * len(triples))()
     keep = []
+    size = _word_bytes(m)
     for i, (f, g, h) in enumerate(triples):
         if not (f.is_cuda and g.is_cuda and h.is_cuda):
             raise ValueError("conv_batched operands must be CUDA tensors")
         if not (f.is_contiguous() and g.is_contiguous() and h.is_contiguous()):
             raise ValueError("conv_batched operands must be contiguous")
+        if f.element_size() != size or g.element_size() != size or h.element_size() != size:
+            raise TypeError(f"conv_batched operands modulo {m} must be {8 * size}-bit words")
         if f.numel() != g.numel() or f.numel() != h.numel():
             raise ValueError("f, g, h of one convolution must have the same length")
         arr[i] = ConvDesc(f.data_ptr(), g.data_ptr(), h.data_ptr(), f.numel(), 0)
@@ -390,7 +398,7 @@ class BatchPlan:
     """``ntt_batch_plan``: an uneven batch of convolutions modulo m."""
 
     def __init__(self, m: int, triples):
-        self.descs, self._keep = _descs(triples)
+        self.descs, self._keep = _descs(m, triples)
         h = ctypes.c_void_p()
         _check(lib().ntt_batch_plan(m, ctypes.cast(self.descs, ctypes.c_void_p), len(triples), ctypes.byref(h)),
                "ntt_batch_plan")
@@ -420,12 +428,16 @@ def ntt_batch_plan(m: int, triples) -> BatchPlan:
 
 def conv_batched(m: int, triples, stream=None):
     """Convolve a list of (f, g, h) CUDA tensors of power-of-two lengths mod m."""
-    arr, _keep = _descs(triples)
+    arr, _keep = _descs(m, triples)
     _check(lib().conv_batched(m, ctypes.cast(arr, ctypes.c_void_p), len(triples), _stream(stream)), "conv_batched")
 
 
 def ntt_check_range(plan: Plan, x: torch.Tensor, stream=None) -> int:
     """Number of words of x that are >= m (synchronous)."""
+    if x.element_size() * 8 != plan.word_bits:
+        raise TypeError(f"x: dtype {x.dtype} does not match {plan.word_bits}-bit words")
+    if not (x.is_cuda or x.is_pinned()) or not x.is_contiguous():
+        raise ValueError("x must be a contiguous CUDA tensor")
     bad = ctypes.c_uint64(0)
     st = lib().ntt_check_range(plan.handle, x.data_ptr(), x.numel(), ctypes.byref(bad), _stream(stream))
     if st not in (NTT_OK, 4):
@@ -463,6 +475,12 @@ class Server:
         """Queue h = f (*) g; tensors that must stay alive until wait() returns
         (pinned or CUDA tensors run in place, pageable ones are staged
         through the pool).  Returns the request id."""
+        n, size = f.numel(), _word_bytes(self.m)
+        for name, t in (("f", f), ("g", g), ("h", h)):
+            if t.element_size() != size:
+                raise TypeError(f"{name}: dtype {t.dtype} does not match {8 * size}-bit words")
+            if not t.is_contiguous() or t.numel() < n:
+                raise ValueError(f"{name} must be a contiguous tensor of {n} words")
         rid = ctypes.c_uint64(0)
         st = lib().ntt_server_submit(self.handle, f.data_ptr(), g.data_ptr(), h.data_ptr(), f.numel(),
                                      ctypes.byref(rid))

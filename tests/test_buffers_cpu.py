@@ -105,3 +105,43 @@ def test_plain_work_buffer(plan, calls):
     for work in (Buf(4 * N), Buf(4 * N, torch.float64)):
         ntt.conv_circular_plain(plan, x, x, out, work, stream=0)
     assert calls == ["conv_circular_plain"] * 2
+
+
+@pytest.mark.parametrize("m,dtype,wrong", [(13631489, torch.int32, torch.int64), (70525124609, torch.int64, torch.int32)])
+def test_batch_operands_of_another_word_size_are_rejected(calls, m, dtype, wrong):
+    ok = Buf(N, dtype)
+    for i in range(3):
+        triple = [ok, ok, ok]
+        triple[i] = Buf(N, wrong)
+        for make in (ntt.conv_batched, ntt.BatchPlan):
+            with pytest.raises(TypeError):
+                make(m, [(ok, ok, ok), tuple(triple)])
+    assert calls == []
+    ntt.conv_batched(m, [(ok, ok, ok)], stream=0)
+    assert calls == ["conv_batched"]
+
+
+@pytest.mark.parametrize("m,dtype,wrong", [(13631489, torch.int32, torch.int16), (70525124609, torch.int64, torch.int32)])
+def test_server_operands_that_do_not_fit_are_rejected(calls, m, dtype, wrong):
+    srv = ntt.Server.__new__(ntt.Server)
+    srv.handle, srv.m = ctypes.c_void_p(), m
+    ok = Buf(N, dtype, cuda=False)
+    bad = [Buf(N, wrong, cuda=False), Buf(N, dtype, cuda=False, contiguous=False)]
+    for i in range(3):
+        for b in bad + [Buf(N // 2, dtype, cuda=False)] * (i > 0):
+            ops = [ok, ok, ok]
+            ops[i] = b
+            with pytest.raises((ValueError, TypeError)):
+                srv.submit(*ops)
+    assert calls == []
+    srv.submit(ok, ok, ok)
+    srv.submit(ok, Buf(2 * N, dtype), Buf(2 * N, dtype))
+    assert calls == ["ntt_server_submit"] * 2
+
+
+def test_range_check_of_another_word_size_is_rejected(plan, calls):
+    for x in (Buf(N, torch.int16), Buf(N, torch.int64), Buf(N, contiguous=False), Buf(N, cuda=False)):
+        with pytest.raises((ValueError, TypeError)):
+            ntt.ntt_check_range(plan, x, stream=0)
+    assert calls == []
+    assert ntt.ntt_check_range(plan, Buf(N + 3), stream=0) == 0 and calls == ["ntt_check_range"]
