@@ -199,14 +199,17 @@ ntt_status conv_batched(uint64_t m, const ntt_conv_desc *descs, size_t count, nt
 /* Build a reusable execution plan for an uneven batch: groups the
  * descriptors by length, builds the per-length plans and device work lists,
  * picks each length's schedule (from the autotune table when one is loaded),
- * and allocates the scratch it needs.  Synchronous.  The descriptor array is
+ * and allocates the scratch it needs: for lengths on the split path up to 1 GB
+ * for each of at most two internal streams (more only where one pair or the
+ * length's own wave needs it), the plans' own waves alone where memory is
+ * short; held until the batch plan is destroyed.  Synchronous.  The descriptor array is
  * copied; the pointers it holds must stay valid while the batch plan is
  * executed. */
 ntt_status ntt_batch_plan(uint64_t m, const ntt_conv_desc *descs, size_t count, ntt_batch_t *out);
 
 /* Enqueue every convolution of the batch plan on `stream` (the persistent
  * launch of the short lengths and the other length classes' launches run on
- * two forked internal streams joined back into `stream`).  Capturable in a
+ * up to three forked internal streams joined back into `stream`).  Capturable in a
  * CUDA graph. */
 ntt_status ntt_batch_exec(ntt_batch_t batch, ntt_stream_t stream);
 

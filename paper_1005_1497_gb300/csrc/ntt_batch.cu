@@ -18,8 +18,7 @@
 #include "ntt_internal.h"
 #include "ntt_count.h"
 #include "ntt_launch.h"
-
-
+#include "host_sched.h"
 
 namespace {
 
@@ -199,32 +198,27 @@ extern "C" ntt_status ntt_batch_plan(uint64_t m, const ntt_conv_desc *descs, siz
             load[k] += 1;
         }
     const int K = own + (load[0] > 0) + (load[1] > 0);
-    // Scratch of the split classes, as the plans' own may be in use elsewhere:
-    // one piece per stream, used by its classes in turn, for every pair of a
-    // class in one wave up to SCRATCH_MAX (fewer, fuller launches: measured on
-    // GB300, 143 x 2^19 in waves of 64 pairs 721 us, in one 679 us), for the
-    // plan's own wave at least, and that where memory is short.
-    constexpr size_t SCRATCH_MAX = (size_t)1 << 30;
+    // Scratch of the split classes, as the plans' own may be in use elsewhere.
+    std::vector<ntt::ScratchClass> split;
+    std::vector<BatchClass *> owner;
+    for (auto &c : b->classes) {
+        ntt_plan_info_t info;
+        ntt_plan_get_info(c.plan, &info);
+        if (!info.four_step) continue;
+        split.push_back(ntt::ScratchClass{c.stream, 2 * ((size_t)1 << c.L) * elt, c.count, info.wave, 0});
+        owner.push_back(&c);
+    }
     b->scratch.assign(K, nullptr);
-    for (int k = 0; k < K; ++k)
-        for (size_t limit = SCRATCH_MAX;; limit = 0) {
-            size_t bytes = 0;
-            for (auto &c : b->classes) {
-                ntt_plan_info_t info;
-                ntt_plan_get_info(c.plan, &info);
-                if (c.stream != k || !info.four_step) continue;
-                const size_t per_pair = 2 * ((size_t)1 << c.L) * elt;
-                c.wave = (uint32_t)std::min<size_t>(std::max<size_t>(info.wave, limit / per_pair), c.count);
-                bytes = std::max(bytes, c.wave * per_pair);
-            }
-            if (bytes == 0) break;
-            if (ntt::dev_alloc(&b->scratch[k], bytes)) {
-                for (auto &c : b->classes)
-                    if (c.stream == k) c.scratch = b->scratch[k];
-                break;
-            }
-            if (limit == 0) return bail(ntt_fail(NTT_ERR_OOM, "ntt_batch_plan: scratch"));
-        }
+    auto alloc = [](size_t bytes) {
+        void *p;
+        return ntt::dev_alloc(&p, bytes) ? p : nullptr;
+    };
+    if (!ntt::take_scratch(split, b->scratch, alloc, [](void *p) { cudaFree(p); }))
+        return bail(ntt_fail(NTT_ERR_OOM, "ntt_batch_plan: scratch"));
+    for (size_t i = 0; i < split.size(); ++i) {
+        owner[i]->scratch = b->scratch[split[i].stream];
+        owner[i]->wave = split[i].wave;
+    }
     b->streams.resize(K);
     b->done.resize(K);
     for (int i = 0; i < K; ++i) {
