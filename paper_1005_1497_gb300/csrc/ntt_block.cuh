@@ -27,17 +27,19 @@
 // 4096 x 2^14 418 -> 400 us (with the staged loads that the smaller table
 // makes room for: 380 us), 301 x 2^13 of 64-bit words 67.4 -> 59.4 us.
 //
-// Bounds (m < 2^B / 128).  Forward: inputs < m; the unit butterflies of
-// levels 0, 1, 2 leave at most 8m, every later level adds 2m: below 26m for
-// N <= 2^14.  A block product sums four products of such values (c_j g is a
-// Shoup product, < 2m): T < 2704 m^2 < 2^(2B - 2), and Montgomery's
-// reduction leaves T / 2^B + m < 23m.  Inverse: 46m and 92m after the two
-// levels with unit butterflies, 2m more for each of the other ten: at most
-// 112m, below the word.  The last factor 2^BB N^{-1} 2^B (Shoup) takes any
-// word and brings N'^{-1} and Montgomery's 2^B.
-// Roomy 64-bit moduli (r64, m < 2^48; N <= 2^13): products below 13m, so 8m +
-// 8 13m = 112m forward, T < 4 112^2 m^2 < 2^112, Montgomery's result below
-// 2m, and 71m + 9 13m < 2^8 m < 2^56 inverse.
+// Bounds (m < 2^B / 128; the static_asserts below follow them level by
+// level).  Forward: inputs < m; unit butterflies at node 0 of levels 0, 1, 2,
+// the others' products add 2m: below 26m for N <= 2^14 (lazy_forward).  A
+// block product sums four products of such values (c_j g is a Shoup product,
+// < 2m): T < 2704 m^2 < 2^(2B - 2), and Montgomery's reduction leaves T / 2^B
+// + m < 23m.  Inverse: 46m and 92m after the two levels with unit
+// butterflies, 2m more for each of the other ten: at most 112m, below the
+// word.  The last factor 2^BB N^{-1} 2^B (Shoup) takes any word and brings
+// N'^{-1} and Montgomery's 2^B.
+// Roomy 64-bit moduli (r64, m < 2^48; N <= 2^13): products below 13m.  A
+// twiddled node of levels 1 and 2 reaches 15m and 28m, so 132m forward; T <
+// 69696 m^2 < 2^113, Montgomery's result below 3m (the 23m of the others is
+// what the unit butterfly adds); 92m + 9 13m = 209m < 2^8 m < 2^56 inverse.
 #pragma once
 
 #include "ntt_core.cuh"
@@ -48,6 +50,20 @@ constexpr int BB = 2;                        // levels left out; blocks of 2^BB 
 // Lengths below 2^BLOCK_LMIN keep the complete transform (a thread then
 // holds fewer than two blocks).
 constexpr int BLOCK_LMIN = BB + 1;
+
+// Bound of the inverse's `levels` levels, in multiples of m: unit butterflies
+// on values below 23m and 46m at levels 0 and 1, products below P m.
+__host__ __device__ constexpr int lazy_inverse(int levels, int P)
+{
+    int b = 23;
+    for (int l = 0; l < levels; ++l) b = l < 2 && 2 * b > b + P ? 2 * b : b + P;
+    return b;
+}
+// T / 2^B + m for four products of values below F m, m < 2^(B - room), in multiples of m (rounded up)
+__host__ __device__ constexpr long long lazy_product(long long F, int room) { return ((4 * F * F) >> room) + 2; }
+static_assert(lazy_forward(14 - BB, 2, 2) == 26 && lazy_product(26, 7) <= 23 && lazy_inverse(14 - BB, 2) == 112, "m < 2^B / 128, N <= 2^14");
+static_assert(lazy_forward(13 - BB, 2, ROOMY_M2) == 132 && lazy_product(132, 64 - ROOMY_BITS) <= 3 && lazy_inverse(13 - BB, ROOMY_M2) == 209 &&
+              209 < 1 << (56 - ROOMY_BITS), "r64, N <= 2^13");
 
 template <typename W> struct Wide;
 template <> struct Wide<uint32_t> { using T = uint64_t; };

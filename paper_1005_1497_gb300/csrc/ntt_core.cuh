@@ -352,13 +352,27 @@ __device__ __forceinline__ void stage_twiddles(const W *__restrict__ tw, W *stw,
     }
 }
 
+// Lazy bound of the forward tree on inputs < m, in multiples of m: products
+// below P m, node 0 without a product up to level `unit`.  Level 0 leaves
+// < 2m.  Node 0 of level d <= unit takes values below 2^d m and leaves both
+// its halves (the next level's nodes 0 and 1) below 2^(d+1) m; a butterfly
+// with a product adds P m.
+__host__ __device__ constexpr int lazy_forward(int levels, int unit, int P)
+{
+    int node0 = 2, others = 2;
+    for (int d = 1; d < levels; ++d) {
+        const int left = d <= unit ? 2 * node0 : node0 + P;
+        others = others + P > left ? others + P : left;
+        node0 = left;
+    }
+    return node0 > others ? node0 : others;
+}
+static_assert(lazy_forward(14, 4, 2) == 50, "natural-order transforms, N <= 2^14: below the word for m < 2^B / 128");
+static_assert(lazy_forward(13, 4, ROOMY_M2) == 158 && 158 < 1 << (56 - ROOMY_BITS), "r64, N <= 2^13: below 2^56, what its product takes");
+
 // One forward level: element bit b = lo_P + JJ, global level L-1-b.
 // Z0: the node base of this pass is known to be 0 (first pass of a whole
-// sequence), so node 0 has the twiddle 1.  Bound note: inputs < m, level 0
-// leaves < 2m and every node-0 butterfly of levels 1..4 doubles the bound
-// (< 2^(d+1) m after level d), the others add 2m: at most 32m + 2m (L - 5)
-// after the forward, below 50m for L <= 14 (r64: 32m + 13m (L - 5), below
-// 2^8 m < 2^56 for L <= 13).
+// sequence), so node 0 has the twiddle 1 (bounds: lazy_forward).
 // UN: the last level whose node 0 skips the product.
 template <typename W, int L, int LR, int P, int JJ, int NS, int TWS, bool Z0 = false, int UN = 4>
 __device__ __forceinline__ void fwd_level(W (&v)[NS][Geo<W, LR>::R], uint32_t xbase,
