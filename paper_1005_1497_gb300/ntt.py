@@ -125,7 +125,10 @@ def _stream(stream) -> int:
     if stream is None:
         if not torch.cuda.is_initialized():
             torch.cuda.init()
-        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+        try:
+            return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+        except AttributeError:              # (private calls: a torch without them)
+            return torch.cuda.current_stream().cuda_stream
     if isinstance(stream, torch.cuda.Stream):
         return stream.cuda_stream
     return int(stream)

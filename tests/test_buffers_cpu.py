@@ -145,3 +145,12 @@ def test_range_check_of_another_word_size_is_rejected(plan, calls):
             ntt.ntt_check_range(plan, x, stream=0)
     assert calls == []
     assert ntt.ntt_check_range(plan, Buf(N + 3), stream=0) == 0 and calls == ["ntt_check_range"]
+
+
+def test_current_stream_without_the_raw_handle(monkeypatch):
+    """A torch without the private calls that read the handle directly: the public one."""
+    for name in ("_cuda_getCurrentRawStream", "_cuda_getDevice"):
+        monkeypatch.delattr(torch._C, name, raising=False)
+    monkeypatch.setattr(torch.cuda, "is_initialized", lambda: True)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda: SimpleNamespace(cuda_stream=77))
+    assert ntt._stream(None) == 77
