@@ -183,6 +183,24 @@ __device__ __forceinline__ void st_garner(size_t at, const W (&r)[VEC], const W 
     }
 }
 
+// R consecutive words from p, 16 bytes at a time where p allows.
+template <typename W, int R>
+__device__ __forceinline__ void ld_row(const W *p, W (&d)[R])
+{
+    constexpr int VEC = (int)(16 / sizeof(W));
+    auto all = [&](bool wide) {
+#pragma unroll
+        for (int k = 0; k < R; k += VEC) {
+            W t[VEC];
+            ld_vec<W, VEC>(p + k, t, wide);
+#pragma unroll
+            for (int e = 0; e < VEC; ++e) d[k + e] = t[e];
+        }
+    };
+    if (((uintptr_t)p & 15u) == 0) all(true);
+    else all(false);
+}
+
 // Fused convolution of whole sequences (L <= LR_max), persistent.  The block
 // stages the twiddle table in shared memory once.  Per pair, f and g are
 // transformed together (one set of twiddle reads serves both) through shared
@@ -224,6 +242,16 @@ __device__ __forceinline__ void conv_fused_body(const RowArgs<W> &a, long long b
     };
     constexpr uint32_t INB = X::IN64 ? 8u : (uint32_t)sizeof(W);     // bytes per input element
     constexpr bool STAGE = SH::STAGE && !X::IN64 && SRC != 2;
+    // One thread per pair: its sequences are consecutive words, read and
+    // written by 16-byte accesses.  By single words every access of a warp
+    // touches 32 lines and counts on the L1 cache to bring the other words of
+    // their sectors once, which the persistent launch, whose longest length
+    // takes most of the SM's shared memory, leaves no room for: measured on
+    // GB300, a batch plan of 1000 pairs of each of 2^0 .. 2^10 by single words
+    // 77 us, by 16 bytes 40 (61 when that launch took 64 KB less), 3000 of 2^0
+    // .. 2^9 of 64-bit words 85 and 76 (76); 37450 x 2^5 alone 11 us (30 for
+    // the complete transform by single words).
+    constexpr bool WHOLE = T == 1 && SH::BLOCKS && std::is_same<X, NoExact>::value;
     W *B = reinterpret_cast<W *>(smem_raw + SH::next) + (size_t)gid * N;
     using BG = BGeo<W, L>;
     const W *fp, *gp, *fn = nullptr, *gn = nullptr;
@@ -249,15 +277,20 @@ __device__ __forceinline__ void conv_fused_body(const RowArgs<W> &a, long long b
             }
         }
         W v[2][R];
+        if constexpr (WHOLE) {
+            ld_row<W, R>(fp, v[0]);
+            ld_row<W, R>(gp, v[1]);
+        } else {
 #pragma unroll
-        for (int k = 0; k < R; ++k) {
-            const uint32_t x = b0 + ((uint32_t)k << lo0);
-            if constexpr (STAGE) {
-                v[0][k] = B[x];
-                v[1][k] = S[BG::ROWP + x];
-            } else {
-                v[0][k] = ld_elem<X>(fp, x, xa, a.c);
-                v[1][k] = ld_elem<X>(gp, x, xa, a.c);
+            for (int k = 0; k < R; ++k) {
+                const uint32_t x = b0 + ((uint32_t)k << lo0);
+                if constexpr (STAGE) {
+                    v[0][k] = B[x];
+                    v[1][k] = S[BG::ROWP + x];
+                } else {
+                    v[0][k] = ld_elem<X>(fp, x, xa, a.c);
+                    v[1][k] = ld_elem<X>(gp, x, xa, a.c);
+                }
             }
         }
         if constexpr (STAGE) {
@@ -275,6 +308,18 @@ __device__ __forceinline__ void conv_fused_body(const RowArgs<W> &a, long long b
             if constexpr (STAGE) {
                 cp_async_wait();
                 group_sync<T>(gid);
+            }
+            if constexpr (WHOLE) {
+                constexpr int VEC = (int)(16 / sizeof(W));
+                const bool wide = ((uintptr_t)hp & 15u) == 0;
+#pragma unroll
+                for (int k = 0; k < R; k += VEC) {          // VEC positions of one block: consecutive outputs
+                    W t[VEC];
+#pragma unroll
+                    for (int e = 0; e < VEC; ++e) t[e] = canon<W>(v[0][k + e], a.c.cB, a.c.cBp, a.c.m);
+                    st_vec<W, VEC>(hp + block_out<L>((uint32_t)k), t, wide);
+                }
+                continue;
             }
 #pragma unroll
             for (int k = 0; k < R; ++k) {
