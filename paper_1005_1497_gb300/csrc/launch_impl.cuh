@@ -271,10 +271,6 @@ static cudaError_t launch_bitrev(const W *src, W *dst, long long batch, const Mo
         const long long tiles = batch << (L - 10);
         k_bitrev_tiled<W, L, INV><<<(unsigned)tiles, 256, 0, st>>>(src, dst, batch, c);
         return launched();
-    } else if constexpr (L >= 1) {
-        const long long n = batch << L;
-        k_bitrev_out<W, L, INV><<<(unsigned)((n + 255) / 256), 256, 0, st>>>(src, dst, batch, c);
-        return launched();
     } else {
         return cudaErrorInvalidValue;
     }

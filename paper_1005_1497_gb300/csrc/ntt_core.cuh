@@ -503,20 +503,16 @@ __host__ __device__ constexpr int brv_c(int j)
     return r;
 }
 
-// Level l = lo_P + JJ of the inverse on one sequence.  In the first pass
-// (lo = 0) every thread's run starts at entry 0, whose twiddle is 1: those
-// butterflies skip the product.  Bound note: inputs < 2m, level 0 leaves
-// < 4m, the unit butterflies of levels 1..4 double it (< 2^(l+2) m after
-// level l), the others add 2m: at most 64m + 2m (L - 5), below 82m for
-// L <= 14, and the final Shoup reduction accepts any word.
-template <typename W, int LR, int P, int JJ, int TWS>
-__device__ __forceinline__ void dit_level(W (&v)[Geo<W, LR>::R], uint32_t xbase,
-                                          const W *__restrict__ tw, const ModC<W> &c)
+// Level JJ of the inverse on one sequence of a single register pass (lengths
+// without blocks: at most 4).  Every thread's run starts at entry 0, whose
+// twiddle is 1: those butterflies skip the product.  Bound note: inputs < 2m,
+// level 0 leaves < 4m and level 1 at most twice that.
+template <typename W, int LR, int JJ, int TWS>
+__device__ __forceinline__ void dit_level(W (&v)[Geo<W, LR>::R], const W *__restrict__ tw, const ModC<W> &c)
 {
-    using G = Geo<W, LR>;
-    constexpr int R = G::R, lo = G::lo(P);
-    constexpr int l = lo + JJ;
-    if constexpr (l == 0) {
+    static_assert(Geo<W, LR>::NPASS == 1 && LR <= 2, "one pass, two levels");
+    constexpr int R = Geo<W, LR>::R;
+    if constexpr (JJ == 0) {
 #pragma unroll
         for (int k = 0; k < R; ++k) {
             if (k & 1) continue;
@@ -526,21 +522,18 @@ __device__ __forceinline__ void dit_level(W (&v)[Geo<W, LR>::R], uint32_t xbase,
         }
     } else {
         constexpr int CNT = 1 << JJ;                  // distinct twiddles of this level
-        constexpr int CH = (CNT >= 2 && tw_per_chunk<W>() == 2) ? 2 : 1;
-        uint32_t tlo = 0;
-        if constexpr (lo > 0) tlo = __brev(xbase & ((1u << lo) - 1u)) >> (32 - lo);
-        const uint32_t run = tlo << JJ;               // aligned to CNT
+        constexpr int CH = tw_per_chunk<W>() == 2 ? 2 : 1;
 #pragma unroll
         for (int t0 = 0; t0 < CNT; t0 += CH) {
             W z[CH], zp[CH];
-            load_tw<W, CH, TWS>(tw, run, (uint32_t)t0, z, zp);
+            load_tw<W, CH, TWS>(tw, 0u, (uint32_t)t0, z, zp);
 #pragma unroll
             for (int tt = 0; tt < CH; ++tt) {
                 const int j = brv_c<JJ>(t0 + tt);         // register bits below JJ
 #pragma unroll
                 for (int hi = 0; hi < (R >> (JJ + 1)); ++hi) {
                     const int k = (hi << (JJ + 1)) | j;
-                    if (lo == 0 && l <= 4 && t0 + tt == 0) ct_bfly_unit<W>(v[k], v[k | (1 << JJ)], c.m << (l + 1));
+                    if (t0 + tt == 0) ct_bfly_unit<W>(v[k], v[k | (1 << JJ)], c.m << (JJ + 1));
                     else ct_bfly<W>(v[k], v[k | (1 << JJ)], z[tt], zp[tt], c);
                 }
             }
@@ -548,13 +541,12 @@ __device__ __forceinline__ void dit_level(W (&v)[Geo<W, LR>::R], uint32_t xbase,
     }
 }
 
-template <typename W, int LR, int P, int JJ, int TWS>
-__device__ __forceinline__ void dit_levels(W (&v)[Geo<W, LR>::R], uint32_t xbase,
-                                           const W *__restrict__ tw, const ModC<W> &c)
+template <typename W, int LR, int JJ, int TWS>
+__device__ __forceinline__ void dit_levels(W (&v)[Geo<W, LR>::R], const W *__restrict__ tw, const ModC<W> &c)
 {
-    if constexpr (JJ < Geo<W, LR>::nb(P)) {
-        dit_level<W, LR, P, JJ, TWS>(v, xbase, tw, c);
-        dit_levels<W, LR, P, JJ + 1, TWS>(v, xbase, tw, c);
+    if constexpr (JJ < LR) {
+        dit_level<W, LR, JJ, TWS>(v, tw, c);
+        dit_levels<W, LR, JJ + 1, TWS>(v, tw, c);
     }
 }
 
@@ -620,19 +612,6 @@ __device__ __forceinline__ void inv_all(W (&v)[Geo<W, LR>::R], uint32_t rowoff, 
     if constexpr (P > 0) {
         exchange1<W, LR, P, P - 1>(v, S, tau, gid);
         inv_all<W, L, LR, P - 1, TWS>(v, rowoff, tau, S, gid, tw, c);
-    }
-}
-
-// All inverse passes, decimation in time, P = FROM .. 0.
-template <typename W, int LR, int P, int TWS>
-__device__ __forceinline__ void dit_all(W (&v)[Geo<W, LR>::R], uint32_t rowoff, uint32_t tau,
-                                        W *S, int gid, const W *__restrict__ tw, const ModC<W> &c)
-{
-    using G = Geo<W, LR>;
-    dit_levels<W, LR, P, 0, TWS>(v, rowoff + G::base(P, tau), tw, c);
-    if constexpr (P > 0) {
-        exchange1<W, LR, P, P - 1>(v, S, tau, gid);
-        dit_all<W, LR, P - 1, TWS>(v, rowoff, tau, S, gid, tw, c);
     }
 }
 

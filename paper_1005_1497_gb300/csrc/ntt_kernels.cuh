@@ -330,7 +330,7 @@ __device__ __forceinline__ void conv_fused_body(const RowArgs<W> &a, long long b
             fwd_all<W, L, L, 0, 2, TW_SMEM, true>(v, 0u, tau, S, gid, stw, a.c);
 #pragma unroll
             for (int k = 0; k < R; ++k) v[0][k] = pointwise(v[0][k], v[1][k], a.c);
-            dit_all<W, L, last, TW_SMEM>(v[0], 0u, tau, S, gid, stw, a.c);
+            dit_levels<W, L, 0, TW_SMEM>(v[0], stw, a.c);
 #pragma unroll
             for (int k = 0; k < R; ++k)
                 st_out<X>(hp, a.pair0 + rho, N, (N - (uint32_t)k) & (N - 1u), canon<W>(v[0][k], (W)1, a.c.onep, a.c.m), xa, a.c);
@@ -1412,7 +1412,7 @@ __global__ void __launch_bounds__(BLOCK, 1) k_rows_uni(const __grid_constant__ R
 // u2, so the tile is GPC consecutive words of every output run of 2^LC.
 // INV counts the tile's rows by the output residue instead (t = <-u>_N), so
 // that its runs are aligned too.  The factor a.c.ninv is the caller's (see
-// k_bitrev_out).  It saves the bit-reversal pass, a read and a write of every
+// k_bitrev_tiled).  It saves the bit-reversal pass, a read and a write of every
 // word; GPC words of 4 bytes are a 32-byte sector for rows of 2^11 and half
 // of one for 2^12, which L2 merges.
 template <typename W, int L, int LR> struct RowsOutShape {
@@ -1474,21 +1474,7 @@ __global__ void __launch_bounds__(BLOCK, 1) k_rows_out(const __grid_constant__ N
 // Bit-reversal gather of a split-path spectrum: y[u] = X(u) from the tree
 // order (X(brv(x)) at x); INV applies <-u>_N.  The factor c.ninv is the
 // caller's: N^-1 for the inverse, and what undoes the scale of the twist's
-// diagonal.  Canonical outputs.
-template <typename W, int L, bool INV>
-__global__ void k_bitrev_out(const W *__restrict__ src, W *__restrict__ dst, long long batch, ModC<W> c)
-{
-    constexpr uint32_t N = 1u << L;
-    const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= batch << L) return;
-    const long long b = idx >> L;
-    const uint32_t t = (uint32_t)idx & (N - 1u);
-    const uint32_t u = INV ? ((N - t) & (N - 1u)) : t;
-    const uint32_t x = __brev(u) >> (32 - L);
-    dst[idx] = csub<W>(shoup<W>(src[(size_t)b * N + x], c.ninv, c.ninvp, c.m), c.m);
-}
-
-// The same gather, tiled (L >= 10): write an index as (h, m, l) with h and
+// diagonal.  Canonical outputs.  Tiled: write an index as (h, m, l) with h and
 // l of 5 bits, so brv(h, m, l) = (brv l, brv m, brv h).  For one value of m
 // the 32 x 32 elements u = (uh, m, ul) come from x = (brv ul, brv m, brv uh):
 // a block reads them as 32 contiguous source runs (fixed brv ul), passes
