@@ -183,11 +183,15 @@ __device__ __forceinline__ void st_garner(size_t at, const W (&r)[VEC], const W 
     }
 }
 
+// Words per access of one thread's R consecutive words: 16 bytes, or single
+// words where there are fewer.
+template <typename W, int R> __host__ __device__ constexpr int row_vec() { return R * sizeof(W) >= 16 ? (int)(16 / sizeof(W)) : 1; }
+
 // R consecutive words from p, 16 bytes at a time where p allows.
 template <typename W, int R>
 __device__ __forceinline__ void ld_row(const W *p, W (&d)[R])
 {
-    constexpr int VEC = (int)(16 / sizeof(W));
+    constexpr int VEC = row_vec<W, R>();
     auto all = [&](bool wide) {
 #pragma unroll
         for (int k = 0; k < R; k += VEC) {
@@ -197,7 +201,7 @@ __device__ __forceinline__ void ld_row(const W *p, W (&d)[R])
             for (int e = 0; e < VEC; ++e) d[k + e] = t[e];
         }
     };
-    if (((uintptr_t)p & 15u) == 0) all(true);
+    if (((uintptr_t)p & (VEC * sizeof(W) - 1)) == 0) all(true);
     else all(false);
 }
 
@@ -310,7 +314,7 @@ __device__ __forceinline__ void conv_fused_body(const RowArgs<W> &a, long long b
                 group_sync<T>(gid);
             }
             if constexpr (WHOLE) {
-                constexpr int VEC = (int)(16 / sizeof(W));
+                constexpr int VEC = row_vec<W, R>();
                 const bool wide = ((uintptr_t)hp & 15u) == 0;
 #pragma unroll
                 for (int k = 0; k < R; k += VEC) {          // VEC positions of one block: consecutive outputs
@@ -937,12 +941,14 @@ template <typename W, int L> struct NttShape {
     using G = Geo<W, L>;
     static constexpr int GPC = BLOCK / G::T;
     static constexpr size_t rows = TwBytes<W, L>::v, next = rows + (size_t)GPC * G::ROWP * sizeof(W);
-    static constexpr size_t smem = next + (size_t)GPC * G::ROW * sizeof(W);
+    static constexpr size_t smem = G::T == 1 ? rows : next + (size_t)GPC * G::ROW * sizeof(W);
 };
 
-// One transform of the loop both kernels share: the staged sequence through
+// One transform of the loop these kernels share: the staged sequence through
 // the forward tree, the next one's copies issued once every thread of the
-// group has read this one; v in the last pass's layout.
+// group has read this one; v in the last pass's layout.  (The group's first
+// sequence straight into registers, for batches of one sequence per group:
+// 4096 x 2^14 169 -> 176 us, not kept.)
 template <typename W, int L, class Next>
 __device__ __forceinline__ void staged_forward(W (&v)[1][Geo<W, L>::R], const W *B, W *S, uint32_t tau, int gid, const W *stw,
                                                const ModC<W> &c, Next next)
@@ -952,13 +958,9 @@ __device__ __forceinline__ void staged_forward(W (&v)[1][Geo<W, L>::R], const W 
 #pragma unroll
     for (int k = 0; k < G::R; ++k) v[0][k] = B[b0 + ((uint32_t)k << G::lo(0))];
     fwd_pass<W, L, L, 0, 1, TW_SMEM, true>(v, b0, stw, c);
-    if constexpr (G::NPASS > 1) {
-        exchange<W, L, 0, 1, 1>(v, S, tau, gid);
-        next();
-        fwd_all<W, L, L, 1, 1, TW_SMEM, true>(v, 0u, tau, S, gid, stw, c);
-    } else {
-        next();                                             // (one thread per sequence)
-    }
+    exchange<W, L, 0, 1, 1>(v, S, tau, gid);
+    next();
+    fwd_all<W, L, L, 1, 1, TW_SMEM, true>(v, 0u, tau, S, gid, stw, c);
 }
 
 template <typename W, int L, bool INV>
@@ -978,25 +980,56 @@ __global__ void __launch_bounds__(BLOCK, 1) k_ntt_rows(const __grid_constant__ N
     stage_twiddles<W>(a.tw, stw, TwBytes<W, L>::pairs);
     const long long step = (long long)gridDim.x * GPC;
     long long rho = (long long)blockIdx.x * GPC + gid;
-    auto stage = [&](long long r) { if (r < a.batch) stage_seq<W, L, Q>(a.x + (size_t)r * N, B, tau); };
-    stage(rho);
-    cp_async_wait();
-    __syncthreads();
-    W v[1][R];
-    for (; rho < a.batch; rho += step) {
-        staged_forward<W, L>(v, B, S, tau, gid, stw, a.c, [&] { stage(rho + step); });
-        cp_async_wait();                                    // visible after the next two barriers
-        group_sync<T>(gid);
-        scatter_reversed<W, L>(v[0], S, tau);
-        group_sync<T>(gid);
-        // output index t = b0 + k T (a warp's stores are one aligned run);
-        // the inverse takes its value from <-t>_N
-        gather_natural<W, L, INV>(v[0], S, tau);
-        W *yp = a.y + (size_t)rho * N;
+    if constexpr (T == 1) {
+        // One thread per sequence: read and written by 16 bytes, reordered
+        // in registers, the next one loaded ahead.  Measured on GB300 against
+        // staging and reordering in shared memory, whose rows of N words
+        // share banks: 1198373 x 2^3 30.2 -> 12.5 us, 299594 x 2^5 62 -> 20.6;
+        // 64-bit words 1198373 x 2^3 58.7 -> 28.4, 599187 x 2^4 69.4 -> 41.2.
+        constexpr int VEC = row_vec<W, R>();
+        W w[R];
+        if (rho < a.batch) ld_row<W, R>(a.x + (size_t)rho * N, w);
+        __syncthreads();
+        for (; rho < a.batch; rho += step) {
+            W v[1][R];
 #pragma unroll
-        for (int k = 0; k < R; ++k)
-            yp[b0 + ((uint32_t)k << G::lo(0))] = csub<W>(INV ? shoup_full<W>(v[0][k], a.c.ninv, a.c.ninvp, a.c.m)
-                                                             : shoup_one<W>(v[0][k], a.c.onep, a.c.m), a.c.m);
+            for (int k = 0; k < R; ++k) v[0][k] = w[k];
+            if (rho + step < a.batch) ld_row<W, R>(a.x + (size_t)(rho + step) * N, w);
+            fwd_pass<W, L, L, 0, 1, TW_SMEM, true>(v, 0u, stw, a.c);
+            W *yp = a.y + (size_t)rho * N;
+            const bool wide = ((uintptr_t)yp & (VEC * sizeof(W) - 1)) == 0;
+#pragma unroll
+            for (int t0 = 0; t0 < R; t0 += VEC) {
+                W o[VEC];
+#pragma unroll
+                for (int e = 0; e < VEC; ++e) {
+                    const W x = v[0][brv_c<L>(INV ? (R - t0 - e) & (R - 1) : t0 + e)];
+                    o[e] = csub<W>(INV ? shoup_full<W>(x, a.c.ninv, a.c.ninvp, a.c.m) : shoup_one<W>(x, a.c.onep, a.c.m), a.c.m);
+                }
+                st_vec<W, VEC>(yp + t0, o, wide);
+            }
+        }
+    } else {
+        auto stage = [&](long long r) { if (r < a.batch) stage_seq<W, L, Q>(a.x + (size_t)r * N, B, tau); };
+        stage(rho);
+        cp_async_wait();
+        __syncthreads();
+        W v[1][R];
+        for (; rho < a.batch; rho += step) {
+            staged_forward<W, L>(v, B, S, tau, gid, stw, a.c, [&] { stage(rho + step); });
+            cp_async_wait();                                // visible after the next two barriers
+            group_sync<T>(gid);
+            scatter_reversed<W, L>(v[0], S, tau);
+            group_sync<T>(gid);
+            // output index t = b0 + k T (a warp's stores are one aligned run);
+            // the inverse takes its value from <-t>_N
+            gather_natural<W, L, INV>(v[0], S, tau);
+            W *yp = a.y + (size_t)rho * N;
+#pragma unroll
+            for (int k = 0; k < R; ++k)
+                yp[b0 + ((uint32_t)k << G::lo(0))] = csub<W>(INV ? shoup_full<W>(v[0][k], a.c.ninv, a.c.ninvp, a.c.m)
+                                                                 : shoup_one<W>(v[0][k], a.c.onep, a.c.m), a.c.m);
+        }
     }
 }
 
