@@ -547,8 +547,10 @@ extern "C" ntt_status conv_circular_host(ntt_plan_t p, const void *f, const void
     // for).  Measured on GB300, in place against the copies: 1 x 2^10 18
     // against 33 us, 256 x 2^14 (48 MB) 227 against 309, 1024 x 2^14 (192 MB)
     // 796 against 866, 1500 x 2^14 (281 MB) 1150 against 1247, from 384 MB on
-    // within 3%; the shorter lengths, whose kernels stage, 16384 x 2^8 (48 MB)
-    // 263 against 296 but 65536 x 2^8 (192 MB) 1052 against 854.
+    // within 3%; 2^10 .. 2^13 at 100, 200 and 318 MB: 2^10 409, 764, 1179
+    // against 494, 896, 1313, 2^12 431, 830, 1279 against 505, 901, 1309, 2^11
+    // and 2^13 as 2^12; the shorter lengths, whose kernels stage, 16384 x 2^8
+    // (48 MB) 263 against 296 but 65536 x 2^8 (192 MB) 1052 against 854.
     // NTT_HOST_DIRECT (percent) overrides that: its share of the pairs goes in
     // place on its own stream while the copy engines stage the rest.
     const size_t direct_max = (size_t)(p->word == 32 && p->L >= ntt::HOST_LMIN ? 320 : 96) << 20;

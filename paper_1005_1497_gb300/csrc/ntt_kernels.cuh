@@ -882,8 +882,11 @@ __device__ __forceinline__ void persist_item(const PersistArgs<W> &a, const Work
 {
     constexpr int RW = Arith<W>::RB + 5;
     // rows [first, first + count) of the descriptor list; the one-warp body
-    // takes them as a local copy of its arguments with nrows set (it compiles
-    // without spills that way), the column/row body as an explicit bound
+    // takes them as a local copy of its arguments with nrows set, the
+    // column/row body as an explicit bound.  (64-bit words of up to 2^9: 144
+    // bytes of spills where the complete transform had 24, and faster all the
+    // same, on GB300: 61440 pairs of 2^6 .. 2^9 177 -> 166 us, 8192 x 2^9 111
+    // -> 104, 16384 x 2^8 95 -> 90, 1200 pairs 45.6 -> 43.2.)
     if constexpr (L <= RW) {
         RowArgs<W> ra = a.cls[L];
         ra.nrows = w.first + w.count;
@@ -1182,7 +1185,7 @@ __device__ __forceinline__ void col_fwd_levels(W (&v)[1 << (L - LR)], const W *_
 }
 
 // Column kernels run blocks of COLB threads and are bound by memory latency:
-// what counts is how many warps have their loads in flight, so each form has
+// what counts is how many warps have their loads in flight, so the forms have
 // a register cap that sets them.  Measured on GB300 (64 x 2^19 unless said;
 // 128-thread blocks against 256: 2-3%, small batches 6%, less of a last wave
 // is empty):
@@ -1190,7 +1193,8 @@ __device__ __forceinline__ void col_fwd_levels(W (&v)[1 << (L - LR)], const W *_
 //    loaded once): 96 registers, five blocks, 83.8 us, 0.94 of the copy rate
 //    (six, 80 registers and spills: 86.1; four: 84.9);
 //  - otherwise one thread per sequence and column: 64-bit words 84 -> 63 us
-//    at 128 x 2^16 against a loop over f and g.
+//    at 128 x 2^16 against a loop over f and g.  (The 32-bit form's 128 only
+//    bounds what the compiler takes, 127; smaller caps were not compared.)
 constexpr int COLB = 128;
 template <typename W, int NS, bool TWIST> __host__ __device__ constexpr bool cols_both() { return TWIST && NS == 2 && sizeof(W) == 4; }
 template <typename W, bool BOTH, int RC>
