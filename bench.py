@@ -529,7 +529,8 @@ def measure_uniform(name, args, world, rank, local, sub=False):
         "roofline": {"bound": "alu", "achieved": round(alu_ach, 1), "peak": round(alu_peak, 1), "unit": "Gmodmul/s",
                      "frac": round(alu_ach / alu_peak, 4), "traffic": traffic,
                      "peak_src": f"{IMAD_PER_SM_CLK} IMAD/clk/SM x SMs x {sm_max_mhz:.0f} MHz / {SLOTS_PER_MODMUL} "
-                                 f"slots per Shoup product",
+                                 f"slots per Shoup product; achieved counts the complete radix-2 transforms' products "
+                                 f"(lengths from 8 convolve by blocks and issue fewer multiplies)",
                      "kernel": kernel, "launch_ms": round(launch_ms, 4), "launches_per_step": launches_per_step},
         "roofline_hbm": {"bound": "hbm", "achieved": round(hbm_ach, 1), "peak": hbm_peak, "unit": "GB/s",
                          "frac": round(hbm_ach / hbm_peak, 4), "peak_src": f"{peak_src} copy bandwidth",
